@@ -168,7 +168,9 @@ MCLBM_API int mclbm_get_params(const mclbm_ctx* ctx, double* params);
 
 /* Advance every sample by nsteps fused stream+collide steps (Eq. (lbIteration)
  * with the KBC collision Eq. (kbcCollision) and the closed-form stabiliser
- * Eq. (entropyControl)).  Enqueued only.  Errors: INVALID_ARG, CUDA. */
+ * Eq. (entropyControl)).  Calls of several steps on FP32 storage run as one launch that keeps the
+ * lattice planes in work in L2 (the same results; unless mclbm_set_launch has chosen a shape).
+ * Enqueued only.  Errors: INVALID_ARG, CUDA. */
 MCLBM_API int mclbm_step(mclbm_ctx* ctx, int64_t nsteps);
 
 /* Number of steps taken since the last initialisation. */
@@ -308,7 +310,7 @@ MCLBM_API int mclbm_leray_params(const double* X, int32_t M, int32_t transpose, 
  * MCLBM_OPT_EXACT_GAMMA, and only they; vec = the first of the type's list, block 128).
  * Results do not depend on the shape (same arithmetic per node, every operation
  * rounded once in the same order).  mclbm_set_launch sets the shape of every step (under AA
- * streaming, of both parities); mclbm_get_launch reports the shape of pull steps and AA even
+ * streaming, of both parities), each of which is then a launch of its own; mclbm_get_launch reports the shape of pull steps and AA even
  * steps.  Errors: INVALID_ARG (unsupported shape, vec not dividing N, kind 6 on a context
  * without MCLBM_OPT_EXACT_GAMMA or another kind on one with it). */
 MCLBM_API int mclbm_set_launch(mclbm_ctx* ctx, int32_t kind, int32_t vec, int32_t block);

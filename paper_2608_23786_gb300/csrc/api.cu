@@ -332,6 +332,7 @@ int mclbm_create(const mclbm_config* cfg, void* d_pop, size_t pop_bytes, void* d
     c->twiddles_ready = false;
     c->launch = default_launch(cfg->precision, cfg->pattern, cfg->options);
     c->launch_odd = default_launch_odd(cfg->precision, cfg->pattern, cfg->options, cfg->N);
+    c->launch_chosen = false;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
     c->num_sms = sms;
@@ -413,7 +414,9 @@ int mclbm_step(mclbm_ctx* ctx, int64_t nsteps)
 {
     if (!ctx || nsteps < 0) return set_error(MCLBM_ERR_INVALID_ARG, "bad ctx or nsteps < 0");
     MCLBM_ON_DEVICE(ctx->device);
-    for (int64_t s = 0; s < nsteps; ++s) MCLBM_CUDA(launch_step(ctx));
+    int64_t taken = 0;
+    MCLBM_CUDA(launch_march(ctx, nsteps, &taken));
+    for (int64_t s = taken; s < nsteps; ++s) MCLBM_CUDA(launch_step(ctx));
     return MCLBM_OK;
 }
 

@@ -203,6 +203,7 @@ int mclbm_set_launch(mclbm_ctx* ctx, int32_t kind, int32_t vec, int32_t block)
     int st = check_shape(ctx, c);
     if (st != MCLBM_OK) return st;
     ctx->launch = ctx->launch_odd = c;
+    ctx->launch_chosen = true;
     return MCLBM_OK;
 }
 
@@ -215,7 +216,9 @@ int mclbm_set_launch_parity(mclbm_ctx* ctx, int32_t parity, int32_t kind, int32_
 {
     if (!ctx) return set_error(MCLBM_ERR_INVALID_ARG, "ctx is NULL");
     const std::vector<mclbm_ctx*> one{ctx};
-    return set_parity_shape(one, ctx->launch, ctx->launch_odd, parity, LaunchConfig{vec, kind == 1 ? 0 : block, kind});
+    const int st = set_parity_shape(one, ctx->launch, ctx->launch_odd, parity, LaunchConfig{vec, kind == 1 ? 0 : block, kind});
+    if (st == MCLBM_OK) ctx->launch_chosen = true;
+    return st;
 }
 
 int mclbm_get_launch_parity(const mclbm_ctx* ctx, int32_t parity, int32_t* kind, int32_t* vec, int32_t* block)

@@ -53,6 +53,7 @@ struct mclbm_ctx {
     bool twiddles_ready;  // FFT twiddle table computed in the work buffer
     mclbm::LaunchConfig launch;      // stepper variant of pull steps and AA even steps (autotuned or default)
     mclbm::LaunchConfig launch_odd;  // AA odd steps (pull: equal to launch)
+    bool launch_chosen;              // the caller set a shape: every step is a launch of that shape
     int num_sms;
     double grad_ms[4];  // last mclbm_grad: forward, recompute, reverse (adjoint kernels), parameter reduction
 };
@@ -107,6 +108,7 @@ void* lattice_ptr(const mclbm_ctx* c, int which);
 // kernels (launchers return cudaError_t of the launch)
 cudaError_t launch_init(const mclbm_ctx* c, const double* d_params);
 cudaError_t launch_step(mclbm_ctx* c);  // one step of one context; updates cur and steps
+cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken);  // march.cu
 cudaError_t launch_step_with(mclbm_ctx* c, const LaunchConfig& cfg, const LaunchConfig& cfg_odd);
 cudaError_t launch_wait_selftest(mclbm_ctx* c);
 // one step of several levels in one launch; updates each level's cur and steps

@@ -1,0 +1,135 @@
+// Host side of the multi-step kernel (stepper_march.cuh): which calls take it, and the parameters of
+// its order.
+#include "internal.h"
+#include "launch.h"
+#include "level_args.cuh"
+#include "stepper_march.cuh"
+
+namespace mclbm {
+
+cudaError_t launch_march_f32(MarchArgs<float>& a, bool pull, int num_sms, int64_t tiles, cudaStream_t s);
+
+namespace {
+
+// L2 that the tiles in work may take.  GB300's 129 MB also hold lines on their way out: 64^3 ensembles
+// whose lattice fits whole run at full speed up to 100 MB (FP32 AA, copy within L2 13.4 TB/s at 100 MB,
+// 11.6 at 160), so 90 MB is kept for the lattice or for the window.
+constexpr int64_t kL2Bytes = int64_t(90) << 20;
+
+// Tiles between a tile and the ones of the step before that it waits for, per group of warps: the
+// tile in work, the one whose loads are in flight, and the report's way to the hand-out.  Measured at
+// 64^3 x 64 and 128^3 x 32 FP32: 2.5 to 5 within 2% of each other, 2 with the window's edge in sight.
+constexpr int64_t kDistance2 = 7;  // in halves
+
+// Longest launch: updates after which a launch ends and the next begins (about a second).
+constexpr int64_t kMaxUpdates = int64_t(4) << 33;
+
+int ilog2(int64_t v)
+{
+    int l = 0;
+    while ((int64_t(1) << (l + 1)) <= v) ++l;
+    return l;
+}
+
+// Fills in the order of `steps` steps; false where no window of two or more steps fits L2.
+template <class E>
+bool march_order(MarchArgs<E>& a, const mclbm_ctx* c, int vec, int64_t steps)
+{
+    const int64_t tile = (int64_t)kMarchGroup * vec;
+    const int64_t plane = (int64_t)c->N * c->N;
+    const int64_t unit = plane > tile ? plane : tile;
+    const int64_t tiles = (int64_t)c->M * c->n / tile;
+    const int64_t tile_bytes = tile * Q * (int64_t)sizeof(E);
+    const int64_t distance = kDistance2 * c->num_sms * kMarchGroups / 2;
+    a.logT = ilog2(unit / tile);
+    a.logU = ilog2(c->n / unit);
+    // chunks of up to 32 tiles: one plane, or several of a small lattice
+    a.logC = 0;
+    while (a.logC < a.logU && (1u << (a.logC + a.logT)) < 32) ++a.logC;
+    const int64_t ct = int64_t(1) << (a.logC + a.logT);
+    const int64_t chunks = tiles / ct;
+    a.chunks = (unsigned)chunks;
+    a.lanes = 1;
+    a.lag = 0;
+    if (tiles * tile_bytes > kL2Bytes) {
+        // Depth: a pass of `lanes` steps crosses HBM once, so from four on HBM is no longer the bound;
+        // of 4 to 12 take the one that leaves the fewest lanes idle in the last pass, the deepest of
+        // equals; two or three where only they fit.  A chunk's dependences reach one chunk ahead at
+        // the step before, two where a chunk is one unit (its last unit needs the next one).
+        const int64_t reach = a.logC == 0 ? 2 : 1;
+        int64_t best = 0, best_idle = 0;
+        for (int64_t lanes = 12; lanes >= 2 && !(best && lanes < 4); --lanes) {
+            const int64_t lag = (distance + lanes * ct - 1) / (lanes * ct) + reach;
+            if (lanes * lag * ct * tile_bytes > kL2Bytes || chunks < (lanes - 1) * lag + 3) continue;
+            const int64_t idle = (steps + lanes - 1) / lanes * lanes - steps;
+            if (best == 0 || idle < best_idle) {
+                best = lanes;
+                best_idle = idle;
+                a.lag = (unsigned)lag;
+            }
+        }
+        if (best == 0) return false;
+        a.lanes = (unsigned)best;
+    }
+    const int64_t passes = (steps + a.lanes - 1) / a.lanes;
+    const int64_t slots = passes * chunks + (int64_t)(a.lanes - 1) * a.lag;
+    if (tiles * (steps + 1) >= (int64_t)1 << 30 || slots * a.lanes * ct >= (int64_t)1 << 31) return false;
+    a.steps = (unsigned)steps;
+    a.slots = (unsigned)slots;
+    return true;
+}
+
+// Whether `steps` steps of a context run faster in the multi-step kernel than with a launch per step:
+// FP32 storage, whose launch per step is at the HBM bound (FP16 and FP64 storage are bound by
+// arithmetic).  The kernel's start (counters, cooperative launch, fill and drain) costs about 11 us a
+// call; per step it saves 1 to 2 us below 2^16 nodes (4.2 against 3.5 us at 8^3 to 32^3), 3 us at 32^3 x
+// 7 (8.3 against 5.4), 4 us at 64^3 (10.4 against 6.4), and a third of the time from 64^3 x 2 on
+// (64^3 x 64 381 against 273 us, AA 387 against 261; 128^3 x 8 385 against 273).  Three steps: 64^3 x 2
+// AA 47.9 against 38.9 us, 64^3 34.1 against 30.9 us, 32^3 x 3 23.3 against 25.1 us.
+bool march_serves(const mclbm_ctx* c, int64_t steps)
+{
+    if (c->cfg.precision != MCLBM_FP32 || (c->cfg.options & MCLBM_OPT_EXACT_GAMMA) || c->launch_chosen) return false;
+    const int64_t nodes = (int64_t)c->M * c->n;
+    return steps >= (nodes < (1 << 16) ? 12 : (nodes < (1 << 18) ? 6 : 3));
+}
+
+}  // namespace
+
+// Takes steps of a call for `nsteps` steps in the multi-step kernel, where it serves the context;
+// *taken is the number taken (the caller takes the others launch by launch).
+cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
+{
+    *taken = 0;
+    const bool pull = c->cfg.pattern == MCLBM_PULL;
+    const int vec = Q == 19 ? 4 : 2;
+    if (!march_serves(c, pull ? nsteps & ~(int64_t)1 : nsteps)) return cudaSuccess;
+    MarchArgs<float> a;
+    memset(&a, 0, sizeof(a));
+    const int64_t tiles = (int64_t)c->M * c->n / (kMarchGroup * vec);
+    const int64_t updates = (int64_t)c->M * c->n;
+    const int64_t most = (kMaxUpdates / updates > 2 ? kMaxUpdates / updates : 2) & ~(int64_t)1;
+    while (*taken < nsteps) {
+        int64_t k = nsteps - *taken < most ? nsteps - *taken : most;
+        if (pull) k &= ~(int64_t)1;
+        if (k < 2 || !march_order(a, c, vec, k)) break;
+        const size_t cnt_bytes = sizeof(int) * ((size_t)c->M << a.logU);
+        if (cnt_bytes > kPartialBytes) break;
+        a.cnt = (int*)(c->work + c->wl.partial);
+        a.err = (int*)(c->work + c->wl.flag) + 1;
+        fill_level<float>(a.lev, c);
+        a.lev.dst = (float*)lattice_ptr(c, pull ? c->cur : 0);
+        if (pull) a.lev.parity = 1;
+        cudaError_t e = cudaMemsetAsync(a.cnt, 0, cnt_bytes, c->stream);
+        if (e == cudaSuccess) e = launch_march_f32(a, pull, c->num_sms, tiles, c->stream);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {  // part of the GPU only: launch by launch
+            cudaGetLastError();
+            break;
+        }
+        if (e != cudaSuccess) return e;
+        c->steps += k;
+        *taken += k;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace mclbm

@@ -5,6 +5,7 @@
 
 #include "internal.h"
 #include "launch.h"
+#include "level_args.cuh"
 #include "stepper_impl.cuh"
 #include "stepper_staged.cuh"
 
@@ -57,9 +58,6 @@ int grid_for(int64_t total)
     return (int)(b > (int64_t)1 << 30 ? (int64_t)1 << 30 : b);
 }
 
-Geom geom_of(const mclbm_ctx* c) { return Geom{c->N, c->logN, c->n}; }
-int parity_of(const mclbm_ctx* c) { return c->cfg.pattern == MCLBM_AA ? (int)(c->steps & 1) : 0; }
-
 template <class E>
 cudaError_t get_t(const mclbm_ctx* c, int sample, double* d_out)
 {
@@ -74,29 +72,6 @@ cudaError_t set_t(mclbm_ctx* c, int sample, const double* d_in)
     k_set_pops<E><<<grid_for(c->n), kBlock, 0, c->stream>>>((E*)lattice_ptr(c, c->cur), geom_of(c), c->cfg.pattern,
                                                             parity_of(c), sample, d_in);
     return cudaGetLastError();
-}
-
-template <class E>
-void fill_level(LevelArgs<E>& L, const mclbm_ctx* c)
-{
-    if (c->cfg.pattern == MCLBM_PULL) {
-        L.src = (const E*)lattice_ptr(c, c->cur);
-        L.dst = (E*)lattice_ptr(c, 1 - c->cur);
-    } else {
-        L.src = (const E*)lattice_ptr(c, 0);
-        L.dst = (E*)lattice_ptr(c, 0);
-    }
-    L.g = geom_of(c);
-    L.M = c->M;
-    L.parity = parity_of(c);
-    L.omega32 = (float)c->units.omega;
-    L.omega64 = c->units.omega;
-    L.a32 = (float)(2.0 / c->units.omega);
-    L.b32 = (float)(2.0 - 2.0 / c->units.omega);
-    if constexpr (std::is_same<E, double>::value) {
-        L.a64 = 2.0 / c->units.omega;
-        L.b64 = 2.0 - 2.0 / c->units.omega;
-    }
 }
 
 template <class E>

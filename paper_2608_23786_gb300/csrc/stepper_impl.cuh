@@ -86,11 +86,46 @@ struct RawOf<16> {
     using type = uint4;
 };
 
-template <class E, int VEC>
+// Loads of lattice data that other blocks of the same launch write (k_march): generic coherent
+// loads served by L2 (never the non-coherent read-only path), ordered by the "memory" clobber.
+__device__ __forceinline__ unsigned short ld_cg(const unsigned short* p)
+{
+    unsigned short r;
+    asm volatile("ld.global.cg.u16 %0, [%1];" : "=h"(r) : "l"(p) : "memory");
+    return r;
+}
+__device__ __forceinline__ unsigned int ld_cg(const unsigned int* p)
+{
+    unsigned int r;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(r) : "l"(p) : "memory");
+    return r;
+}
+__device__ __forceinline__ uint2 ld_cg(const uint2* p)
+{
+    uint2 r;
+    asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(p) : "memory");
+    return r;
+}
+__device__ __forceinline__ uint4 ld_cg(const uint4* p)
+{
+    uint4 r;
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+                 : "l"(p)
+                 : "memory");
+    return r;
+}
+
+// COH: a coherent load (see ld_cg); otherwise through the read-only path.
+template <class E, int VEC, bool COH = false>
 __device__ __forceinline__ void vload(const E* p, E (&out)[VEC])
 {
     using R = typename RawOf<VEC * sizeof(E)>::type;
-    const R r = __ldg(reinterpret_cast<const R*>(p));
+    R r;
+    if constexpr (COH)
+        r = ld_cg(reinterpret_cast<const R*>(p));
+    else
+        r = __ldg(reinterpret_cast<const R*>(p));
     memcpy(out, &r, sizeof(R));
 }
 
@@ -103,15 +138,12 @@ __device__ __forceinline__ void vstore(E* p, const E (&in)[VEC])
     *reinterpret_cast<R*>(p) = r;
 }
 
-template <class E>
+template <class E, bool COH = false>
 __device__ __forceinline__ E sload(const E* p)
 {
-    return __ldg(p);
-}
-template <>
-__device__ __forceinline__ __half sload<__half>(const __half* p)
-{
-    return __ushort_as_half(__ldg(reinterpret_cast<const unsigned short*>(p)));
+    E v[1];
+    vload<E, 1, COH>(p, v);
+    return v[0];
 }
 
 template <class E>
@@ -371,14 +403,14 @@ __device__ __forceinline__ void gather_all(const E* base, const Geom& g, int x0,
 }
 
 // Store all Q post-collision populations: slot I of the row shifted by SIGN * c_i.
-template <class E, int VEC, int SIGN, bool WRAP = false, int I = 0>
+template <class E, int VEC, int SIGN, bool WRAP = false, bool SWAP = false, int I = 0>
 __device__ __forceinline__ void scatter_rows(E* base, const Geom& g, const RowOffsets& r, int x0, int lane,
                                              const typename Storage<E>::compute (&v)[Q][VEC])
 {
     if constexpr (I < Q) {
-        scatter_row<E, VEC, SIGN * Dir<I>::x, WRAP>(run_at(base, g, I, r, SIGN * Dir<I>::y, SIGN * Dir<I>::z), x0,
+        scatter_row<E, VEC, SIGN * Dir<I>::x, WRAP>(run_at(base, g, SWAP ? Dir<I>::o : I, r, SIGN * Dir<I>::y, SIGN * Dir<I>::z), x0,
                                                      g.N, lane, v[I]);
-        scatter_rows<E, VEC, SIGN, WRAP, I + 1>(base, g, r, x0, lane, v);
+        scatter_rows<E, VEC, SIGN, WRAP, SWAP, I + 1>(base, g, r, x0, lane, v);
     }
 }
 template <class E, int VEC, int I = 0>
@@ -391,12 +423,12 @@ __device__ __forceinline__ void scatter_direct(E* base, const Geom& g, int x0, i
     }
 }
 // SIGN 1: the AA odd step (row offsets); 0: pull, own rows (direct addresses).
-template <class E, int VEC, int SIGN, bool WRAP = false>
+template <class E, int VEC, int SIGN, bool WRAP = false, bool SWAP = false>
 __device__ __forceinline__ void scatter_all(E* base, const Geom& g, int x0, int y, int z, int lane,
                                             const typename Storage<E>::compute (&v)[Q][VEC])
 {
     if constexpr (SIGN != 0)
-        scatter_rows<E, VEC, SIGN, WRAP>(base, g, row_offsets(g, x0, y, z), x0, lane, v);
+        scatter_rows<E, VEC, SIGN, WRAP, SWAP>(base, g, row_offsets(g, x0, y, z), x0, lane, v);
     else
         scatter_direct<E, VEC>(base, g, x0, y, z, lane, v);
 }
@@ -413,7 +445,7 @@ __device__ __forceinline__ void load_own(const E* base, const Geom& g, int64_t n
         for (int k = 0; k < VEC; ++k) v[i][k] = to_c<E>(w[k]);
     }
 }
-template <class E, int VEC>
+template <class E, int VEC, bool SWAP = false>
 __device__ __forceinline__ void store_own_opp(E* base, const Geom& g, int64_t node, const typename Storage<E>::compute (&v)[Q][VEC])
 {
 #pragma unroll
@@ -421,7 +453,7 @@ __device__ __forceinline__ void store_own_opp(E* base, const Geom& g, int64_t no
         E w[VEC];
 #pragma unroll
         for (int k = 0; k < VEC; ++k) w[k] = from_c<E>(v[i][k]);
-        vstore<E, VEC>(base + (int64_t)opp(i) * g.n + node, w);
+        vstore<E, VEC>(base + (int64_t)(SWAP ? i : opp(i)) * g.n + node, w);
     }
 }
 
@@ -493,15 +525,15 @@ struct RunLoc {
     int64_t node;
 };
 
-template <class E, int VEC, int CXI, bool WRAP = false>
+template <class E, int VEC, int CXI, bool WRAP = false, bool COH = false>
 __device__ __forceinline__ void issue_row(const E* run, int x0, int N, int lane, RawRun<E, VEC>& r)
 {
-    vload<E, VEC>(run, r.w);
+    vload<E, VEC, COH>(run, r.w);
     if constexpr (WRAP) {  // the row's lanes rotate: no end element to load
     } else if constexpr (CXI > 0) {
-        if (lane == 0 || x0 == 0) r.edge = sload<E>(run + before_run(x0, N));
+        if (lane == 0 || x0 == 0) r.edge = sload<E, COH>(run + before_run(x0, N));
     } else if constexpr (CXI < 0) {
-        if (lane == 31 || x0 + VEC == N) r.edge = sload<E>(run + after_run<VEC>(x0, N));
+        if (lane == 31 || x0 + VEC == N) r.edge = sload<E, COH>(run + after_run<VEC>(x0, N));
     }
 }
 
@@ -555,47 +587,48 @@ __device__ __forceinline__ void finish_row(const RawRun<E, VEC>& r, int x0, int 
     }
 }
 
-template <class E, int VEC, int FIX, bool WRAP = false, int I = 0>
+template <class E, int VEC, int FIX, bool WRAP = false, bool COH = false, bool SWAP = false, int I = 0>
 __device__ __forceinline__ void issue_rows(const E* base, const Geom& g, const RowOffsets& r, const RunLoc& p,
                                            int lane, RawRun<E, VEC> (&raw)[Q])
 {
     if constexpr (I < Q) {
         const int mode = FIX >= 0 ? FIX : p.mode;
         const bool shift = mode != 1;
-        const int slot = mode == 2 ? Dir<I>::o : I;
+        const int slot = (mode == 2) != SWAP ? Dir<I>::o : I;
         const E* run = run_at(base, g, slot, r, shift ? -Dir<I>::y : 0, shift ? -Dir<I>::z : 0);
         if (shift)
-            issue_row<E, VEC, Dir<I>::x, WRAP>(run, p.x0, g.N, lane, raw[I]);
+            issue_row<E, VEC, Dir<I>::x, WRAP, COH>(run, p.x0, g.N, lane, raw[I]);
         else
-            issue_row<E, VEC, 0>(run, p.x0, g.N, lane, raw[I]);
-        issue_rows<E, VEC, FIX, WRAP, I + 1>(base, g, r, p, lane, raw);
+            issue_row<E, VEC, 0, false, COH>(run, p.x0, g.N, lane, raw[I]);
+        issue_rows<E, VEC, FIX, WRAP, COH, SWAP, I + 1>(base, g, r, p, lane, raw);
     }
 }
-template <class E, int VEC, int FIX, bool WRAP = false, int I = 0>
+template <class E, int VEC, int FIX, bool WRAP = false, bool COH = false, bool SWAP = false, int I = 0>
 __device__ __forceinline__ void issue_direct(const E* base, const Geom& g, const RunLoc& p, int lane,
                                              RawRun<E, VEC> (&raw)[Q])
 {
     if constexpr (I < Q) {
         const int mode = FIX >= 0 ? FIX : p.mode;
         const bool shift = mode != 1;
-        const int slot = mode == 2 ? Dir<I>::o : I;
+        const int slot = (mode == 2) != SWAP ? Dir<I>::o : I;
         const E* run = run_direct(base, g, slot, p.x0, p.y, p.z, shift ? -Dir<I>::y : 0, shift ? -Dir<I>::z : 0);
         if (shift)
-            issue_row<E, VEC, Dir<I>::x, WRAP>(run, p.x0, g.N, lane, raw[I]);
+            issue_row<E, VEC, Dir<I>::x, WRAP, COH>(run, p.x0, g.N, lane, raw[I]);
         else
-            issue_row<E, VEC, 0>(run, p.x0, g.N, lane, raw[I]);
-        issue_direct<E, VEC, FIX, WRAP, I + 1>(base, g, p, lane, raw);
+            issue_row<E, VEC, 0, false, COH>(run, p.x0, g.N, lane, raw[I]);
+        issue_direct<E, VEC, FIX, WRAP, COH, SWAP, I + 1>(base, g, p, lane, raw);
     }
 }
 // FIX 2 (AA odd): row offsets; pull, AA even and mixed launches: direct addresses.
-template <class E, int VEC, int FIX, bool WRAP = false>
+// SWAP: a lattice whose slots of opposite velocities are exchanged (see stepper_march.cuh).
+template <class E, int VEC, int FIX, bool WRAP = false, bool COH = false, bool SWAP = false>
 __device__ __forceinline__ void issue_all(const E* base, const Geom& g, const RunLoc& p, int lane,
                                           RawRun<E, VEC> (&raw)[Q])
 {
     if constexpr (FIX == 2)
-        issue_rows<E, VEC, FIX, WRAP>(base, g, row_offsets(g, p.x0, p.y, p.z), p, lane, raw);
+        issue_rows<E, VEC, FIX, WRAP, COH, SWAP>(base, g, row_offsets(g, p.x0, p.y, p.z), p, lane, raw);
     else
-        issue_direct<E, VEC, FIX, WRAP>(base, g, p, lane, raw);
+        issue_direct<E, VEC, FIX, WRAP, COH, SWAP>(base, g, p, lane, raw);
 }
 
 template <class E, int VEC, int FIX, bool WRAP = false, int I = 0>
