@@ -257,7 +257,7 @@ MCLBM_API int mclbm_w1_restricted(const double* d_a, int32_t MA, const double* d
  * of (u_c(x_i), u_c(x_j)) in R^2 for each component c, summed over c.  Euclidean ground
  * metric, every point pair i <= j, off-diagonal pairs counted twice, divided by G^2.  Each
  * pair is an exact transport problem between uniform empirical measures (1 <= MA, MB <= 1024):
- * for L = lcm(MA, MB) <= 64 an assignment of L atoms per side (atoms repeated L/MA, L/MB
+ * for L = lcm(MA, MB) <= 256 an assignment of L atoms per side (atoms repeated L/MA, L/MB
  * times), one warp per problem; otherwise the transportation problem with integer supply MB/g
  * per atom of A and demand MA/g per atom of B (g = gcd(MA, MB)) by successive shortest paths,
  * one block per problem.  Costs are fixed-point integers from FP32 atoms taken relative to

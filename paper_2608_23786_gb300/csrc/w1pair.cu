@@ -12,10 +12,11 @@
 // costs; the distance of the problem is then the FP64 cost of that plan, recomputed from the FP64
 // atoms.  Two solvers:
 //
-//  - L = lcm(M_A, M_B) <= 64: repeating every atom of A L / M_A times and every atom of B L / M_B
+//  - L = lcm(M_A, M_B) <= 256: repeating every atom of A L / M_A times and every atom of B L / M_B
 //    times gives uniform weights 1/L on both sides without changing the optimum, and an optimal
 //    plan is then a permutation: one warp solves the L x L assignment problem with the
-//    shortest-augmenting-path (Hungarian) method, each lane owning columns lane and lane + 32.
+//    shortest-augmenting-path (Hungarian) method after a column reduction, each lane owning up to
+//    eight columns.
 //  - otherwise (M_A, M_B <= 1024): one block solves the transportation problem directly, with
 //    g = gcd(M_A, M_B), integer supply M_B / g at every atom of A and demand M_A / g at every atom
 //    of B (the plan pi = x / (M_A M_B / g)), by successive shortest paths: rows (atoms of A) are
@@ -26,6 +27,7 @@
 //    memory.  Otherwise the integer flows x_ij (at most min(supply, demand) <= 1024, 16 bits) are
 //    kept in a column-major matrix in the work buffer, one per block in flight.
 #include <cmath>
+#include <cstring>
 #include <string>
 
 #include "internal.h"
@@ -34,8 +36,8 @@ namespace mclbm {
 
 namespace {
 
-constexpr int kPairMaxL = 64;  // largest assignment size (two columns per lane)
-constexpr int kPairWarps = 8;  // warps (problems in flight) per block
+constexpr int kPairMaxL = 256;  // largest assignment of the warp kernel (eight columns per lane)
+constexpr int kPairWarps = 4;   // warps (problems in flight) per block
 constexpr long long kInf = 0x3fffffffffffffffLL;
 
 struct PairProblem {
@@ -103,25 +105,67 @@ __device__ __forceinline__ long long qcost(const float (&x)[K], const float (&y)
     return __float2ll_rn(sqrtf(s) * scale);
 }
 
-// One problem per warp.  Shared memory per warp: row atoms X [L][K] (FP32), row potentials
-// u [L], matched row of each column p [L + 1] (slot L: the virtual column of the row being
-// inserted) and the predecessor column way [L].
+// The fixed-point cost as qcost forms it, without the 64-bit conversion (16 results per SM and clock
+// at best): the float is split at 2^20 by adding and subtracting 1.5 2^23, which rounds to nearest in
+// the low mantissa bits; the high part is exact and even, so the sum rounds as the whole would.
 template <int K>
-__global__ void __launch_bounds__(32 * kPairWarps) k_w1_pairs(const double* __restrict__ A, int MA,
-                                                              const double* __restrict__ B, int MB, int G, int L,
-                                                              int ncomp, int64_t nprob, double* __restrict__ per)
+__device__ __forceinline__ long long qcost_split(const float (&x)[K], const float (&y)[K], float scale)
 {
-    __shared__ float sX[kPairWarps][kPairMaxL][K];
-    __shared__ long long su[kPairWarps][kPairMaxL];
-    __shared__ int sp[kPairWarps][kPairMaxL + 1];
-    __shared__ int sway[kPairWarps][kPairMaxL];
+    float s = 0.f;
+#pragma unroll
+    for (int d = 0; d < K; ++d) {
+        const float e = x[d] - y[d];
+        s = fmaf(e, e, s);
+    }
+    const float c = sqrtf(s) * scale;
+    constexpr float kMagic = 12582912.0f;  // 1.5 2^23
+    constexpr int kMagicBits = 0x4B400000;
+    const float h = __fmaf_rn(c, 9.5367431640625e-7f, kMagic);
+    const float r = __fmaf_rn(__fsub_rn(h, kMagic), -1048576.0f, c);
+    const int hi = __float_as_int(h) - kMagicBits;
+    const int lo = __float_as_int(__fadd_rn(r, kMagic)) - kMagicBits;
+    return (long long)hi * 1048576 + lo;
+}
+
+// One assignment problem of L atoms per side per warp, by shortest augmenting paths: rows are
+// inserted one at a time along a shortest path of reduced costs (Dijkstra over the columns), then the
+// potentials of the scanned columns and their rows are updated.  Lane l owns the columns l + 32 c,
+// c < CPL: atom, potential, distance and predecessor row in registers.  Shared memory per warp: the
+// rows (atom and potential, one or two 16-byte words), and the matchings and predecessors as 16-bit
+// indices.  A scan costs about 45 instructions per column of a lane and two warp-wide minima
+// (redux.sync over the halves of the 64-bit distance), with no barrier; the kernel is bound by their
+// issue and latency, so problems in flight are what counts: one warp each instead of a block of 256
+// threads with five barriers per scan.  On the 8^3 grid (131,328 problems), vector / component-wise,
+// against a block per problem: M = 100 487 / 1506 -> 28.5 / 92 ms, M_A, M_B = 100, 50 455 / 1453 ->
+// 40.5 / 117 ms, M = 128 715 / 2236 -> 44 / 143 ms; against a warp that updated every potential at
+// every scan (L <= 64): M = 64 18.8 / 55 -> 8.4 / 29 ms, M = 4 1.9 / 2.6 -> 1.2 / 1.8 ms.  M = 256 on the
+// 4^3 grid 28.4 / 90 -> 5.7 / 12.5 ms: the line to the block kernel is where a lane's columns no longer
+// fit its registers.
+template <int K>
+struct __align__(16) MatchRow {
+    float x[K];
+    long long u;
+};
+
+__host__ __device__ inline int match_smem(int K, int L)  // bytes per warp
+{
+    const int row = K == 6 ? (int)sizeof(MatchRow<6>) : (int)sizeof(MatchRow<2>);
+    return (row * L + 3 * 2 * L + 15) / 16 * 16;
+}
+
+template <int K, int CPL>
+__global__ void __launch_bounds__(32 * kPairWarps) k_w1_match(const double* __restrict__ A, int MA,
+                                                              const double* __restrict__ B, int MB, int G, int L,
+                                                              int ncomp, int64_t nprob, double* __restrict__ per,
+                                                              int* __restrict__ err)
+{
+    extern __shared__ __align__(16) unsigned char msm[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float(*X)[K] = sX[w];
-    long long* u = su[w];
-    int* p = sp[w];
-    int* way = sway[w];
-    const int ra = L / MA, rb = L / MB;  // repetitions of each atom
-    const int VIRT = L;
+    MatchRow<K>* row = reinterpret_cast<MatchRow<K>*>(msm + w * match_smem(K, L));
+    short* rowcol = reinterpret_cast<short*>(row + L);  // column of each matched row
+    short* pcol = rowcol + L;                           // row of each matched column, else -1
+    short* pred = pcol + L;                             // row before a column on its shortest path
+    const int ra = L / MA, rb = L / MB;                 // repetitions of each atom
     for (int64_t prob = (int64_t)blockIdx.x * kPairWarps + w; prob < nprob; prob += (int64_t)gridDim.x * kPairWarps) {
         PairProblem pb;
         pair_of(prob / ncomp, G, pb.i, pb.j);
@@ -130,25 +174,29 @@ __global__ void __launch_bounds__(32 * kPairWarps) k_w1_pairs(const double* __re
         // ensembles' atoms (in FP64), so that their FP32 values resolve the spread of the
         // ensembles rather than the magnitude of the velocity.
         double cen[K];
+        {
+            double ca[K], cb[K];
 #pragma unroll
-        for (int d = 0; d < K; ++d) cen[d] = 0.0;
-        for (int m = lane; m < MA; m += 32) {
-            double x[K];
-            atom64<K>(A, G, m, pb, x);
+            for (int d = 0; d < K; ++d) ca[d] = cb[d] = 0.0;
+            for (int m = lane; m < MA; m += 32) {
+                double x[K];
+                atom64<K>(A, G, m, pb, x);
 #pragma unroll
-            for (int d = 0; d < K; ++d) cen[d] += x[d] / MA;
-        }
-        for (int m = lane; m < MB; m += 32) {
-            double x[K];
-            atom64<K>(B, G, m, pb, x);
+                for (int d = 0; d < K; ++d) ca[d] += x[d];
+            }
+            for (int m = lane; m < MB; m += 32) {
+                double x[K];
+                atom64<K>(B, G, m, pb, x);
 #pragma unroll
-            for (int d = 0; d < K; ++d) cen[d] += x[d] / MB;
-        }
+                for (int d = 0; d < K; ++d) cb[d] += x[d];
+            }
+            const double ia = 0.5 / MA, ib = 0.5 / MB;
 #pragma unroll
-        for (int d = 0; d < K; ++d) {
+            for (int d = 0; d < K; ++d) {
+                cen[d] = ca[d] * ia + cb[d] * ib;
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) cen[d] += __shfl_xor_sync(0xffffffffu, cen[d], off);
-            cen[d] *= 0.5;
+                for (int off = 16; off > 0; off >>= 1) cen[d] += __shfl_xor_sync(0xffffffffu, cen[d], off);
+            }
         }
         // rows: atoms of A (row r is sample r / ra); columns: atoms of B (column s is sample s / rb)
         float amax = 0.f;
@@ -157,30 +205,32 @@ __global__ void __launch_bounds__(32 * kPairWarps) k_w1_pairs(const double* __re
             atom64<K>(A, G, r / ra, pb, x);
 #pragma unroll
             for (int d = 0; d < K; ++d) {
-                X[r][d] = (float)(x[d] - cen[d]);
-                amax = fmaxf(amax, fabsf(X[r][d]));
+                const float f = (float)(x[d] - cen[d]);
+                row[r].x[d] = f;
+                amax = fmaxf(amax, fabsf(f));
             }
-            u[r] = 0;
+            row[r].u = 0;
+            rowcol[r] = pcol[r] = -1;
         }
-        float y[2][K];
-        long long v[2], minv[2];
-        bool used[2], mine[2];
-        int col[2];
+        float y[CPL][K];
+        long long v[CPL], dist[CPL];
+        int from[CPL];
+        unsigned mine = 0;  // the lane's columns, as bits
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            col[q] = lane + 32 * q;
-            mine[q] = col[q] < L;
-            if (mine[q]) {
+        for (int c = 0; c < CPL; ++c) {
+            const int col = lane + 32 * c;
+#pragma unroll
+            for (int d = 0; d < K; ++d) y[c][d] = 0.f;
+            if (col < L) {
+                mine |= 1u << c;
                 double x[K];
-                atom64<K>(B, G, col[q] / rb, pb, x);
+                atom64<K>(B, G, col / rb, pb, x);
 #pragma unroll
                 for (int d = 0; d < K; ++d) {
-                    y[q][d] = (float)(x[d] - cen[d]);
-                    amax = fmaxf(amax, fabsf(y[q][d]));
+                    y[c][d] = (float)(x[d] - cen[d]);
+                    amax = fmaxf(amax, fabsf(y[c][d]));
                 }
             }
-            v[q] = 0;
-            if (mine[q]) p[col[q]] = -1;
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
@@ -188,80 +238,108 @@ __global__ void __launch_bounds__(32 * kPairWarps) k_w1_pairs(const double* __re
         // room for the potentials (sums of at most L costs) in 64 bits
         const float scale = amax > 0.f ? 1099511627776.0f / (2.0f * sqrtf((float)K) * amax) : 1.0f;
         __syncwarp();
-        for (int i = 0; i < L; ++i) {
-            if (lane == 0) p[VIRT] = i;
+        // Column reduction: v = the column's smallest cost, and a column takes the row of that cost
+        // where the row is still free (the lowest column of several).  It halves the scans at K = 6,
+        // M = 100 (1104 -> 574 and 100 passes over the rows without a warp-wide minimum).
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                minv[q] = kInf;
-                used[q] = false;
+        for (int c = 0; c < CPL; ++c) {
+            v[c] = kInf;
+            from[c] = 0;
+        }
+        for (int r = 0; r < L; ++r) {
+            float x[K];
+#pragma unroll
+            for (int d = 0; d < K; ++d) x[d] = row[r].x[d];
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+                const long long q = qcost_split<K>(x, y[c], scale);
+                if (q < v[c]) {
+                    v[c] = q;
+                    from[c] = r;
+                }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+            const int col = lane + 32 * c;
+            const bool wants = col < L && rowcol[from[c]] < 0;
+            const unsigned same = __match_any_sync(0xffffffffu, wants ? from[c] : -1 - lane);
+            if (wants && __ffs(same) - 1 == lane) {
+                rowcol[from[c]] = (short)col;
+                pcol[col] = (short)from[c];
             }
             __syncwarp();
-            int j0 = VIRT;
-            bool found = false;  // a free column was reached (always within i + 1 scans)
+        }
+        bool failed = false;
+        for (int r0 = 0; r0 < L && !failed; ++r0) {
+            if (rowcol[r0] >= 0) continue;
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) dist[c] = kInf;
+            unsigned open = mine;  // columns not yet scanned
+            int i = r0, jstar = -1;
+            long long dcur = 0;
             for (int guard = 0; guard <= L; ++guard) {
-                const int i0 = p[j0];
-                const long long ui0 = u[i0];
+                float x[K];
+#pragma unroll
+                for (int d = 0; d < K; ++d) x[d] = row[i].x[d];
+                const long long base = dcur - row[i].u;
                 long long best = kInf;
-                int bj = VIRT;
+                int bc = 0;
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    if (mine[q] && !used[q]) {
-                        float x[K];
-#pragma unroll
-                        for (int d = 0; d < K; ++d) x[d] = X[i0][d];
-                        const long long cur = qcost<K>(x, y[q], scale) - ui0 - v[q];
-                        if (cur < minv[q]) {
-                            minv[q] = cur;
-                            way[col[q]] = j0;
-                        }
-                        if (minv[q] < best || (minv[q] == best && col[q] < bj)) {
-                            best = minv[q];
-                            bj = col[q];
-                        }
+                for (int c = 0; c < CPL; ++c) {
+                    const long long cand = base + qcost_split<K>(x, y[c], scale) - v[c];
+                    const bool is_open = (open >> c) & 1u;
+                    if (is_open && cand < dist[c]) {
+                        dist[c] = cand;
+                        from[c] = i;
+                    }
+                    if (is_open && dist[c] < best) {
+                        best = dist[c];
+                        bc = c;
                     }
                 }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    const long long ob = __shfl_xor_sync(0xffffffffu, best, off);
-                    const int oj = __shfl_xor_sync(0xffffffffu, bj, off);
-                    if (ob < best || (ob == best && oj < bj)) {
-                        best = ob;
-                        bj = oj;
-                    }
-                }
-                const long long delta = best;
-                // potentials: used columns (and the virtual column) raise the potential of their
-                // row, the others lower their reduced distance
-                if (lane == 0) u[i] += delta;
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    if (!mine[q]) continue;
-                    if (used[q]) {
-                        u[p[col[q]]] += delta;
-                        v[q] -= delta;
-                    } else {
-                        minv[q] -= delta;
-                    }
-                }
-                __syncwarp();
-                j0 = bj;
-                if (j0 >= VIRT) break;
-                if (p[j0] < 0) {
-                    found = true;
+                // the closest open column: minimum of the high words, then of the low words
+                const unsigned hi = (unsigned)(best >> 32), lo = (unsigned)best;
+                const unsigned mhi = __reduce_min_sync(0xffffffffu, hi);
+                const unsigned mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
+                const int wl = __ffs(__ballot_sync(0xffffffffu, hi == mhi && lo == mlo)) - 1;
+                dcur = (long long)(((unsigned long long)mhi << 32) | mlo);
+                if (dcur >= kInf) break;  // nothing reachable: reported below
+                const int j = 32 * __shfl_sync(0xffffffffu, bc, wl) + wl;
+                i = pcol[j];
+                if (i < 0) {
+                    jstar = j;
                     break;
                 }
+                if (lane == wl) open &= ~(1u << bc);
+            }
+            if (jstar < 0) {
+                failed = true;
+                break;
+            }
+            // potentials: scanned columns v -= d* - d, their rows u += d* - d, and the new row u += d*
+            const unsigned scanned = mine & ~open;
 #pragma unroll
-                for (int q = 0; q < 2; ++q)
-                    if (col[q] == j0) used[q] = true;
+            for (int c = 0; c < CPL; ++c) {
+                const int col = lane + 32 * c;
+                if ((scanned >> c) & 1u) {
+                    const long long delta = dcur - dist[c];
+                    v[c] -= delta;
+                    row[pcol[col]].u += delta;
+                }
+                if ((mine >> c) & 1u && ((scanned >> c) & 1u || col == jstar)) pred[col] = (short)from[c];
             }
             __syncwarp();
-            // augment along the predecessor columns back to the virtual column
-            if (lane == 0 && found) {
-                int jj = j0;
-                for (int guard = 0; guard <= L && jj != VIRT; ++guard) {
-                    const int j1 = way[jj];
-                    p[jj] = p[j1];
-                    jj = j1;
+            if (lane == 0) {  // augment along the path back to r0 (at most L columns)
+                row[r0].u += dcur;
+                int j = jstar;
+                for (int guard = 0; guard <= L; ++guard) {
+                    const int ri = pred[j];
+                    const int jn = rowcol[ri];
+                    pcol[j] = (short)ri;
+                    rowcol[ri] = (short)j;
+                    if (ri == r0) break;
+                    j = jn;
                 }
             }
             __syncwarp();
@@ -269,16 +347,21 @@ __global__ void __launch_bounds__(32 * kPairWarps) k_w1_pairs(const double* __re
         // W1 of the problem: mean FP64 cost of the matched pairs
         double s = 0.0;
 #pragma unroll
-        for (int q = 0; q < 2; ++q)
-            if (mine[q] && p[col[q]] >= 0) s += cost64<K>(A, B, G, p[col[q]] / ra, col[q] / rb, pb);
+        for (int c = 0; c < CPL; ++c) {
+            const int col = lane + 32 * c;
+            if (col < L && pcol[col] >= 0) s += cost64<K>(A, B, G, pcol[col] / ra, col / rb, pb);
+        }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) per[prob] = s / L;
+        if (lane == 0) {
+            per[prob] = s / L;
+            if (failed) atomicExch(err, 1);
+        }
         __syncwarp();
     }
 }
 
-// ---- transportation problems beyond the warp kernel: one block per problem -----------------
+// ---- transportation problems beyond the warp kernel (L > 256): one block per problem -----------------
 constexpr int kTpMaxM = 1024;          // atoms per side
 constexpr int kTpThreads = 256;        // threads per block
 constexpr int kTpWarps = kTpThreads / 32;
@@ -687,7 +770,7 @@ PairWork pair_work(int MA, int MB, int G, int vector)
     w.flows = (w.err + 16 + 255) / 256 * 256;
     const int g = gcd_int(MA, MB);
     const int64_t L = (int64_t)MA / g * MB;
-    const bool general = L > kPairMaxL && MA != MB;
+    const bool general = L > 64 && MA != MB;
     const size_t fstride = ((size_t)MA * MB + 7) / 8 * 8;  // elements per block, as in the kernel
     w.bytes = w.flows + (general ? (size_t)kTpGeneralBlocks * fstride * sizeof(unsigned short) : 0);
     return w;
@@ -729,21 +812,39 @@ int mclbm_w1_2pt(const double* d_a, int32_t MA, const double* d_b, int32_t MB, i
     int dev = 0, sms = 0;
     MCLBM_CUDA(cudaGetDevice(&dev));
     MCLBM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    MCLBM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     if (L <= kPairMaxL) {
-        int64_t blocks = (nprob + kPairWarps - 1) / kPairWarps;
-        if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
+        auto launch = [&](auto kernel, int K) -> cudaError_t {
+            const int smem = kPairWarps * match_smem(K, (int)L);
+            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e != cudaSuccess) return e;
+            int per_sm = 0;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * kPairWarps, smem);
+            if (e != cudaSuccess) return e;
+            if (per_sm < 1) return cudaErrorInvalidConfiguration;
+            int64_t blocks = (nprob + kPairWarps - 1) / kPairWarps;
+            if (blocks > (int64_t)sms * per_sm) blocks = (int64_t)sms * per_sm;
+            kernel<<<(unsigned)blocks, 32 * kPairWarps, smem, s>>>(d_a, MA, d_b, MB, G, (int)L, ncomp, nprob, per, err);
+            return cudaGetLastError();
+        };
+        cudaError_t e;
         if (vector)
-            k_w1_pairs<6><<<(unsigned)blocks, 32 * kPairWarps, 0, s>>>(d_a, MA, d_b, MB, G, (int)L, ncomp, nprob, per);
+            e = L <= 32    ? launch(k_w1_match<6, 1>, 6)
+                : L <= 64  ? launch(k_w1_match<6, 2>, 6)
+                : L <= 128 ? launch(k_w1_match<6, 4>, 6)
+                           : launch(k_w1_match<6, 8>, 6);
         else
-            k_w1_pairs<2><<<(unsigned)blocks, 32 * kPairWarps, 0, s>>>(d_a, MA, d_b, MB, G, (int)L, ncomp, nprob, per);
-        MCLBM_CUDA(cudaGetLastError());
+            e = L <= 32    ? launch(k_w1_match<2, 1>, 2)
+                : L <= 64  ? launch(k_w1_match<2, 2>, 2)
+                : L <= 128 ? launch(k_w1_match<2, 4>, 2)
+                           : launch(k_w1_match<2, 8>, 2);
+        MCLBM_CUDA(e);
     } else {
         const bool match = MA == MB;
         const int K = vector ? 6 : 2;
         const int smem = tp_layout(MA, MB, K).total;
         const int supply = MB / g, demand = MA / g;
         unsigned short* flows = match ? nullptr : (unsigned short*)(wb + pw.flows);
-        MCLBM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
         auto launch = [&](auto kernel) -> cudaError_t {
             cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e != cudaSuccess) return e;
@@ -769,10 +870,13 @@ int mclbm_w1_2pt(const double* d_a, int32_t MA, const double* d_b, int32_t MB, i
     k_pair_partials<<<kPairParts, kSumThreads, 0, s>>>(per, G, ncomp, nprob, chunk, partial);
     k_pair_total<<<1, 32, 0, s>>>(partial, kPairParts, 1.0 / ((double)G * G), total);
     MCLBM_CUDA(cudaGetLastError());
-    int h_err = 0;
-    MCLBM_CUDA(cudaMemcpyAsync(W, total, sizeof(double), cudaMemcpyDeviceToHost, s));
-    if (L > kPairMaxL) MCLBM_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    // the total and the error word lie 32 doubles apart: one copy brings both
+    double h_total[33];
+    MCLBM_CUDA(cudaMemcpyAsync(h_total, total, sizeof(h_total), cudaMemcpyDeviceToHost, s));
     MCLBM_CUDA(cudaStreamSynchronize(s));
+    *W = h_total[0];
+    int h_err = 0;
+    memcpy(&h_err, &h_total[32], sizeof(int));
     if (h_err)
         return set_error(MCLBM_ERR_NONFINITE, "a transport search found no column with open demand (non-finite atoms?)");
     return MCLBM_OK;
