@@ -359,7 +359,7 @@ __device__ __forceinline__ void collide_run(typename Storage<E>::compute (&v)[Q]
             if constexpr (Storage<E>::shifted)
                 kbc_shifted<float, Ar>(t, omega, L.a32, L.b32);
             else
-                kbc_raw(t, omega, (C)L.a64, (C)L.b64);
+                kbc_raw(t, omega, L.a64, L.b64);
 #pragma unroll
             for (int i = 0; i < Q; ++i) v[i][k] = t[i];
         }
