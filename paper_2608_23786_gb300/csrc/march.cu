@@ -8,6 +8,7 @@
 namespace mclbm {
 
 cudaError_t launch_march_f32(MarchArgs<float>& a, bool pull, int num_sms, int64_t tiles, cudaStream_t s);
+cudaError_t launch_march_f16(MarchArgs<__half>& a, bool pull, int num_sms, int64_t tiles, cudaStream_t s);
 
 namespace {
 
@@ -79,31 +80,34 @@ bool march_order(MarchArgs<E>& a, const mclbm_ctx* c, int vec, int64_t steps)
     return true;
 }
 
-// Whether `steps` steps of a context run faster in the multi-step kernel than with a launch per step:
-// FP32 storage, whose launch per step is at the HBM bound (FP16 and FP64 storage are bound by
-// arithmetic).  The kernel's start (counters, cooperative launch, fill and drain) costs about 11 us a
-// call; per step it saves 1 to 2 us below 2^16 nodes (4.2 against 3.5 us at 8^3 to 32^3), 3 us at 32^3 x
-// 7 (8.3 against 5.4), 4 us at 64^3 (10.4 against 6.4), and a third of the time from 64^3 x 2 on
-// (64^3 x 64 381 against 273 us, AA 387 against 261; 128^3 x 8 385 against 273).  Three steps: 64^3 x 2
-// AA 47.9 against 38.9 us, 64^3 34.1 against 30.9 us, 32^3 x 3 23.3 against 25.1 us.
+// Whether `steps` steps of a context run faster in the multi-step kernel than with a launch per step.
+// The kernel's start (counters, cooperative launch, fill and drain) costs about 11 us a call.
+//
+// FP32 storage, whose launch per step is at the HBM bound: per step the kernel saves 1 to 2 us below
+// 2^16 nodes (4.2 against 3.5 us at 8^3 to 32^3), 3 us at 32^3 x 7 (8.3 against 5.4), 4 us at 64^3 (10.4
+// against 6.4), and a third of the time from 64^3 x 2 on (64^3 x 64 381 against 273 us, AA 387 against
+// 261; 128^3 x 8 385 against 273).  Three steps: 64^3 x 2 AA 47.9 against 38.9 us, 64^3 34.1 against 30.9
+// us, 32^3 x 3 23.3 against 25.1 us.
+//
+// FP16 storage is bound by arithmetic, in a kernel with twice the nodes per thread (65 against 78 GLUPS
+// at 64^3 x 64): here only what is bound by launches and latency, 6.2 against 3.1 to 3.5 us per step up
+// to 32^3, 64^3 8.3 against 5.3, 64^3 x 4 18.5 against 16.4 (D3Q27 64^3 x 2 14.4 against 13.7 us).
+// FP64 storage is bound by its arithmetic from 32^3 on.
 bool march_serves(const mclbm_ctx* c, int64_t steps)
 {
-    if (c->cfg.precision != MCLBM_FP32 || (c->cfg.options & MCLBM_OPT_EXACT_GAMMA) || c->launch_chosen) return false;
+    if (c->cfg.precision == MCLBM_FP64 || (c->cfg.options & MCLBM_OPT_EXACT_GAMMA) || c->launch_chosen) return false;
     const int64_t nodes = (int64_t)c->M * c->n;
+    if (c->cfg.precision == MCLBM_FP16) return steps >= 6 && nodes <= (Q == 19 ? 1 << 20 : 1 << 19);
     return steps >= (nodes < (1 << 16) ? 12 : (nodes < (1 << 18) ? 6 : 3));
 }
 
-}  // namespace
-
-// Takes steps of a call for `nsteps` steps in the multi-step kernel, where it serves the context;
-// *taken is the number taken (the caller takes the others launch by launch).
-cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
+template <class E>
+cudaError_t march_t(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
 {
-    *taken = 0;
+    constexpr bool f32 = std::is_same<E, float>::value;
     const bool pull = c->cfg.pattern == MCLBM_PULL;
-    const int vec = Q == 19 ? 4 : 2;
-    if (!march_serves(c, pull ? nsteps & ~(int64_t)1 : nsteps)) return cudaSuccess;
-    MarchArgs<float> a;
+    const int vec = Q == 19 || !f32 ? 4 : 2;
+    MarchArgs<E> a;
     memset(&a, 0, sizeof(a));
     const int64_t tiles = (int64_t)c->M * c->n / (kMarchGroup * vec);
     const int64_t updates = (int64_t)c->M * c->n;
@@ -116,11 +120,15 @@ cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
         if (cnt_bytes > kPartialBytes) break;
         a.cnt = (int*)(c->work + c->wl.partial);
         a.err = (int*)(c->work + c->wl.flag) + 1;
-        fill_level<float>(a.lev, c);
-        a.lev.dst = (float*)lattice_ptr(c, pull ? c->cur : 0);
+        fill_level<E>(a.lev, c);
+        a.lev.dst = (E*)lattice_ptr(c, pull ? c->cur : 0);
         if (pull) a.lev.parity = 1;
         cudaError_t e = cudaMemsetAsync(a.cnt, 0, cnt_bytes, c->stream);
-        if (e == cudaSuccess) e = launch_march_f32(a, pull, c->num_sms, tiles, c->stream);
+        if (e != cudaSuccess) return e;
+        if constexpr (f32)
+            e = launch_march_f32(a, pull, c->num_sms, tiles, c->stream);
+        else
+            e = launch_march_f16(a, pull, c->num_sms, tiles, c->stream);
         if (e == cudaErrorCooperativeLaunchTooLarge) {  // part of the GPU only: launch by launch
             cudaGetLastError();
             break;
@@ -130,6 +138,17 @@ cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
         *taken += k;
     }
     return cudaSuccess;
+}
+
+}  // namespace
+
+// Takes steps of a call for `nsteps` steps in the multi-step kernel, where it serves the context;
+// *taken is the number taken (the caller takes the others launch by launch).
+cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
+{
+    *taken = 0;
+    if (!march_serves(c, c->cfg.pattern == MCLBM_PULL ? nsteps & ~(int64_t)1 : nsteps)) return cudaSuccess;
+    return c->cfg.precision == MCLBM_FP32 ? march_t<float>(c, nsteps, taken) : march_t<__half>(c, nsteps, taken);
 }
 
 }  // namespace mclbm

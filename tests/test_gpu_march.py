@@ -1,4 +1,4 @@
-"""Calls of several steps on FP32 storage (one launch of the multi-step kernel) against the same steps
+"""Calls of several steps on FP32 and (small) FP16 storage (one launch of the multi-step kernel) against the same steps
 taken one call at a time (a launch per step): the same bits, for both streaming patterns, one and
 several tiles per plane, several planes per tile, windows and whole lattices in L2, even and odd
 step counts and a state at an odd step."""
@@ -15,8 +15,8 @@ def _lib():
     mclbm.load(build_if_missing=True)
 
 
-def _pair(N, M, **kw):
-    return [Ensemble(N, M, Re=12.5 * N, Ma=1.6 / max(N, 32), precision="fp32", **kw).init() for _ in range(2)]
+def _pair(N, M, precision="fp32", **kw):
+    return [Ensemble(N, M, Re=12.5 * N, Ma=1.6 / max(N, 32), precision=precision, **kw).init() for _ in range(2)]
 
 
 def _same(a, b):
@@ -32,6 +32,17 @@ def _same(a, b):
                                        (128, 2, 7), (256, 1, 5)])
 def test_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
     a, b = _pair(N, M, pattern=pattern, lattice=lattice)
+    a.step(steps)
+    for _ in range(steps):
+        b.step(1)
+    _same(a, b)
+
+
+@pytest.mark.parametrize("lattice", [19, 27])
+@pytest.mark.parametrize("pattern", ["pull", "aa"])
+@pytest.mark.parametrize("N,M,steps", [(8, 1, 7), (16, 3, 6), (32, 7, 9), (64, 2, 6)])
+def test_fp16_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
+    a, b = _pair(N, M, "fp16", pattern=pattern, lattice=lattice)
     a.step(steps)
     for _ in range(steps):
         b.step(1)
