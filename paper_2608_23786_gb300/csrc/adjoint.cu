@@ -30,6 +30,7 @@ namespace {
 
 constexpr int kBlock = 128;
 constexpr int kGradChunks = 64;  // blocks per sample in the parameter reduction
+static_assert(kBlock * kGradChunks % 1024 == 0, "k_param_grad: a thread keeps its x (N <= 1024)");
 
 __device__ __forceinline__ void xyz(const Geom& g, int64_t node, int& x, int& y, int& z)
 {
@@ -283,6 +284,76 @@ __global__ void __launch_bounds__(kRunBlock) k_adjoint_async(const E* __restrict
     cp_async_wait<0>();
 }
 
+// Sums of per-velocity values over the opposite pairs, by weight class: m0 = sum w v (rest included),
+// m1_a = sum w c_a v and, with SECOND, m2 = sum w c_a c_b v (xx, yy, zz, xy, xz, yz).  One weight per
+// class instead of one per velocity: GB300's FP64 units set the time of the kernels that use it.
+template <bool SECOND>
+__device__ __forceinline__ void class_moments(const double (&v)[Q], double w0, double w1, double w2, double w3,
+                                              double& m0, double (&m1)[3], double (&m2)[6])
+{
+    double s[(Q - 1) / 2], d[(Q - 1) / 2];
+#pragma unroll
+    for (int p = 0; p < (Q - 1) / 2; ++p) {
+        s[p] = v[2 * p + 1] + v[2 * p + 2];
+        d[p] = v[2 * p + 1] - v[2 * p + 2];
+    }
+    // pairs: +-x, +-y, +-z, xy(++), xy(+-), xz(++), xz(+-), yz(++), yz(+-), (+++), (++-), (+-+), (+--)
+    const double exy = s[3] + s[4], exz = s[5] + s[6], eyz = s[7] + s[8];
+    m0 = w0 * v[0] + w1 * (s[0] + s[1] + s[2]) + w2 * (exy + exz + eyz);
+    m1[0] = w1 * d[0] + w2 * ((d[3] + d[4]) + (d[5] + d[6]));
+    m1[1] = w1 * d[1] + w2 * ((d[3] - d[4]) + (d[7] + d[8]));
+    m1[2] = w1 * d[2] + w2 * ((d[5] - d[6]) + (d[7] - d[8]));
+    if constexpr (SECOND) {
+        m2[0] = w1 * s[0] + w2 * (exy + exz);
+        m2[1] = w1 * s[1] + w2 * (exy + eyz);
+        m2[2] = w1 * s[2] + w2 * (exz + eyz);
+        m2[3] = w2 * (s[3] - s[4]);
+        m2[4] = w2 * (s[5] - s[6]);
+        m2[5] = w2 * (s[7] - s[8]);
+    }
+#ifdef MCLBM_D3Q27
+    const double c01 = s[9] + s[10], c23 = s[11] + s[12], a01 = d[9] + d[10], a23 = d[11] + d[12];
+    const double cs = w3 * (c01 + c23);
+    m0 += cs;
+    m1[0] += w3 * (a01 + a23);
+    m1[1] += w3 * (a01 - a23);
+    m1[2] += w3 * ((d[9] - d[10]) + (d[11] - d[12]));
+    if constexpr (SECOND) {
+        const double m01 = s[9] - s[10], m23 = s[11] - s[12];
+        m2[0] += cs;
+        m2[1] += cs;
+        m2[2] += cs;
+        m2[3] += w3 * (c01 - c23);
+        m2[4] += w3 * (m01 + m23);
+        m2[5] += w3 * (m01 - m23);
+    }
+#endif
+}
+
+// rho, 1 / rho and u (lattice units) of f(x) in FP64
+template <class E>
+__device__ __forceinline__ void moments_by_class(const E* sample, const Geom& g, int x, int y, int z, double& rho, double& rinv,
+                                          double (&u)[3])
+{
+    double v[Q], j[3], none[6];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const E e = sample[pre_loc(g, kPull, 0, i, x, y, z)];
+        if constexpr (Storage<E>::shifted)
+            v[i] = (double)to_c<E>(e);
+        else
+            v[i] = e;
+    }
+    if constexpr (Storage<E>::shifted) {
+        class_moments<false>(v, weight<double>(0), weight<double>(1), weight<double>(7), weight<double>(Q - 1), rho, j, none);
+        rho += 1.0;
+    } else {
+        class_moments<false>(v, 1.0, 1.0, 1.0, 1.0, rho, j, none);
+    }
+    rinv = rcp64(rho);
+    for (int a = 0; a < 3; ++a) u[a] = j[a] * rinv;
+}
+
 // rho and u (lattice units) of f(x) in FP64
 template <class E>
 __device__ __forceinline__ void moments64(const E* sample, const Geom& g, int x, int y, int z, double& rho, double (&u)[3])
@@ -300,7 +371,8 @@ __device__ __forceinline__ void moments64(const E* sample, const Geom& g, int x,
     for (int a = 0; a < 3; ++a) u[a] = j[a] / r;
 }
 
-// Seed lambda^T = dJ/df^T.  dJ/du_phys(x) is given per node by g_u ([3][n] FP64, one sample) or,
+// Seed lambda^T = dJ/df^T (its FP32 rounding enters the reverse sweep, which amplifies a last bit where
+// Dh is small: the order of its operations stays).  dJ/du_phys(x) is given per node by g_u ([3][n] FP64, one sample) or,
 // when g_u is null, is the kinetic-energy derivative u_phys / N^3.  With u_phys = s j / rho:
 // dJ/df_q = sum_a dJ/du_phys_a s (c_qa - u_a) / rho.
 template <class E, class C>
@@ -344,7 +416,9 @@ __global__ void k_curl(const double* __restrict__ u, double* __restrict__ w, Geo
 }
 
 // Parameter gradient partials: per sample and block, 24 sums of
-// G_a(x) (U_lat / U_c) / 8 a_i(2x) a_j(2y) a_k(2z),  G_a = sum_q lambda_q d f^eq_q / d u_a.
+// G_a(x) (U_lat / U_c) / 8 a_i(2x) a_j(2y) a_k(2z),  G_a = sum_q lambda_q d f^eq_q / d u_a.  Bound by
+// the FP64 units: about 200 operations and conversions per node against 500 with G summed velocity by
+// velocity and 24 products per node (64^3 x 16: 3.57 -> 1.52 ms).
 template <class E, class C>
 __global__ void __launch_bounds__(kBlock) k_param_grad(const E* __restrict__ state0, const C* __restrict__ lam0,
                                                        const double* __restrict__ trig, Geom g, double coef,
@@ -354,36 +428,45 @@ __global__ void __launch_bounds__(kBlock) k_param_grad(const E* __restrict__ sta
     const int m = blockIdx.y;
     const E* smp = state0 + (int64_t)m * Q * g.n;
     const C* lm = lam0 + (int64_t)m * Q * g.n;
-    double acc[24];
+    // a thread's nodes have one x (the stride is a multiple of N): it sums G_a a_j(2y) a_k(2z) and applies
+    // a_i(2x) at the end
+    double yz[12];
 #pragma unroll
-    for (int k = 0; k < 24; ++k) acc[k] = 0.0;
+    for (int k = 0; k < 12; ++k) yz[k] = 0.0;
     for (int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; node < g.n; node += (int64_t)gridDim.x * blockDim.x) {
         int x, y, z;
         xyz(g, node, x, y, z);
-        double rho, u[3];
-        moments64<E>(smp, g, x, y, z, rho, u);
-        double G[3] = {0, 0, 0};
+        double rho, rinv, u[3];
+        moments_by_class<E>(smp, g, x, y, z, rho, rinv, u);
+        // G_a = rho sum_q w_q lambda_q (3 c_a + 9 (c.u) c_a - 3 u_a)
+        double l[Q], l0, l1[3], l2[6];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const double l = (double)lm[(int64_t)q * g.n + node];
-            const double cu = cx(q) * u[0] + cy(q) * u[1] + cz(q) * u[2];
-            const double rw = rho * weight<double>(q) * l;
-            G[0] += rw * (3.0 * cx(q) + 9.0 * cu * cx(q) - 3.0 * u[0]);
-            G[1] += rw * (3.0 * cy(q) + 9.0 * cu * cy(q) - 3.0 * u[1]);
-            G[2] += rw * (3.0 * cz(q) + 9.0 * cu * cz(q) - 3.0 * u[2]);
-        }
-        const double ax[2] = {trig[4 * x + 2], trig[4 * x + 3]};
+        for (int q = 0; q < Q; ++q) l[q] = (double)lm[(int64_t)q * g.n + node];
+        class_moments<true>(l, weight<double>(0), weight<double>(1), weight<double>(7), weight<double>(Q - 1), l0, l1, l2);
+        const double r3 = 3.0 * rho;
+        double G[3];
+        G[0] = r3 * (l1[0] + 3.0 * (l2[0] * u[0] + l2[3] * u[1] + l2[4] * u[2]) - u[0] * l0);
+        G[1] = r3 * (l1[1] + 3.0 * (l2[3] * u[0] + l2[1] * u[1] + l2[5] * u[2]) - u[1] * l0);
+        G[2] = r3 * (l1[2] + 3.0 * (l2[4] * u[0] + l2[5] * u[1] + l2[2] * u[2]) - u[2] * l0);
         const double ay[2] = {trig[4 * y + 2], trig[4 * y + 3]};
         const double az[2] = {trig[4 * z + 2], trig[4 * z + 3]};
 #pragma unroll
-        for (int al = 0; al < 3; ++al)
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int k = 0; k < 2; ++k) {
+                const double p = ay[j] * az[k];
 #pragma unroll
-                for (int j = 0; j < 2; ++j)
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) acc[8 * al + 4 * i + 2 * j + k] += G[al] * (ax[i] * ay[j] * az[k]);
+                for (int al = 0; al < 3; ++al) yz[4 * al + 2 * j + k] += G[al] * p;
+            }
     }
+    const int x = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & (g.N - 1));
+    double acc[24];
+#pragma unroll
+    for (int al = 0; al < 3; ++al)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int jk = 0; jk < 4; ++jk) acc[8 * al + 4 * i + jk] = trig[4 * x + 2 + i] * yz[4 * al + jk];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < 24; ++k) {
@@ -570,11 +653,13 @@ int run_grad(mclbm_ctx* c, int objective, int64_t nsteps, int K, char* buf, size
     double recompute_ms = 0, adjoint_ms = 0;
     pe.mark(0, c->stream);
     // ---- forward with checkpoints every K steps
-    for (int64_t t = 0; t < nsteps; ++t) {
-        if (t % K == 0)
-            MCLBM_CUDA(cudaMemcpyAsync(buf + L.ckpt + (size_t)(t / K) * L.lattice, lattice_ptr(c, c->cur), L.lattice,
-                                       cudaMemcpyDeviceToDevice, c->stream));
-        MCLBM_CUDA(launch_step(c));
+    for (int64_t t = 0; t < nsteps; t += K) {
+        MCLBM_CUDA(cudaMemcpyAsync(buf + L.ckpt + (size_t)(t / K) * L.lattice, lattice_ptr(c, c->cur), L.lattice,
+                                   cudaMemcpyDeviceToDevice, c->stream));
+        const int64_t k = K < nsteps - t ? K : nsteps - t;
+        int64_t taken = 0;
+        MCLBM_CUDA(launch_march(c, k, &taken));
+        for (; taken < k; ++taken) MCLBM_CUDA(launch_step(c));
     }
     if (nsteps == 0)
         MCLBM_CUDA(cudaMemcpyAsync(buf + L.ckpt, lattice_ptr(c, c->cur), L.lattice, cudaMemcpyDeviceToDevice, c->stream));
