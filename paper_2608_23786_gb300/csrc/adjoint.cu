@@ -10,7 +10,7 @@
 //           f^0 = f^eq(rho_0, u_0), u_0 = (U_lat/U_c)(u_det + s(X)), s linear in X.
 // Storage:  checkpoints of the whole lattice every K steps, and for the segment being
 //           reversed the K - 1 intermediate lattices recomputed from its checkpoint
-//           (states cannot all be kept).  lambda is kept in natural layout
+//           (states cannot all be kept; the last segment's are kept by the forward run).  lambda is kept in natural layout
 //           [sample][i][node] in the arithmetic of the stepper (FP32 or FP64).
 #include <cuda_fp16.h>
 
@@ -653,10 +653,28 @@ int run_grad(mclbm_ctx* c, int objective, int64_t nsteps, int K, char* buf, size
     double recompute_ms = 0, adjoint_ms = 0;
     pe.mark(0, c->stream);
     // ---- forward with checkpoints every K steps
+    // the states t0 + 1 .. t1 - 1 of the segment that starts at checkpoint j, in the segment buffer
+    auto trajectory = [&](int64_t j, int64_t states) -> cudaError_t {
+        const char* ck = buf + L.ckpt + (size_t)j * L.lattice;
+        int64_t done = 0;
+        cudaError_t e = launch_march_trajectory(c, ck, buf + L.seg, L.lattice, states, &done);
+        for (; e == cudaSuccess && done < states; ++done)
+            e = launch_pull_explicit(c, done == 0 ? ck : buf + L.seg + (size_t)(done - 1) * L.lattice,
+                                     buf + L.seg + (size_t)done * L.lattice);
+        return e;
+    };
     for (int64_t t = 0; t < nsteps; t += K) {
         MCLBM_CUDA(cudaMemcpyAsync(buf + L.ckpt + (size_t)(t / K) * L.lattice, lattice_ptr(c, c->cur), L.lattice,
                                    cudaMemcpyDeviceToDevice, c->stream));
         const int64_t k = K < nsteps - t ? K : nsteps - t;
+        if (t + k == nsteps && k > 1) {
+            // the last segment keeps its states (the reverse sweep starts there: nothing to recompute);
+            // its last step ends in the context
+            MCLBM_CUDA(trajectory(t / K, k - 1));
+            MCLBM_CUDA(launch_pull_explicit(c, buf + L.seg + (size_t)(k - 2) * L.lattice, lattice_ptr(c, c->cur)));
+            c->steps += k;
+            break;
+        }
         int64_t taken = 0;
         MCLBM_CUDA(launch_march(c, k, &taken));
         for (; taken < k; ++taken) MCLBM_CUDA(launch_step(c));
@@ -686,8 +704,7 @@ int run_grad(mclbm_ctx* c, int objective, int64_t nsteps, int K, char* buf, size
             return t == t0 ? ck : buf + L.seg + (size_t)(t - t0 - 1) * L.lattice;
         };
         pe.mark(2, c->stream);
-        for (int64_t t = t0 + 1; t < t1; ++t)
-            MCLBM_CUDA(launch_pull_explicit(c, state_at(t - 1), (void*)state_at(t)));
+        if (j < L.nckpt - 1) MCLBM_CUDA(trajectory(j, t1 - t0 - 1));
         pe.mark(3, c->stream);
         for (int64_t t = t1 - 1; t >= t0; --t) {
             MCLBM_CUDA(adjoint_step(c, state_at(t), lam_a, lam_b));

@@ -109,6 +109,8 @@ void* lattice_ptr(const mclbm_ctx* c, int which);
 cudaError_t launch_init(const mclbm_ctx* c, const double* d_params);
 cudaError_t launch_step(mclbm_ctx* c);  // one step of one context; updates cur and steps
 cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken);  // march.cu
+cudaError_t launch_march_trajectory(mclbm_ctx* c, const void* src, void* dst, size_t hop_bytes, int64_t nsteps,
+                                    int64_t* taken);
 cudaError_t launch_step_with(mclbm_ctx* c, const LaunchConfig& cfg, const LaunchConfig& cfg_odd);
 cudaError_t launch_wait_selftest(mclbm_ctx* c);
 // one step of several levels in one launch; updates each level's cur and steps

@@ -7,8 +7,8 @@
 
 namespace mclbm {
 
-cudaError_t launch_march_f32(MarchArgs<float>& a, bool pull, int num_sms, int64_t tiles, cudaStream_t s);
-cudaError_t launch_march_f16(MarchArgs<__half>& a, bool pull, int num_sms, int64_t tiles, cudaStream_t s);
+cudaError_t launch_march_f32(MarchArgs<float>& a, int mode, int num_sms, int64_t tiles, cudaStream_t s);
+cudaError_t launch_march_f16(MarchArgs<__half>& a, int mode, int num_sms, int64_t tiles, cudaStream_t s);
 
 namespace {
 
@@ -101,11 +101,12 @@ bool march_serves(const mclbm_ctx* c, int64_t steps)
     return steps >= (nodes < (1 << 16) ? 12 : (nodes < (1 << 18) ? 6 : 3));
 }
 
+// Takes `nsteps` steps in mode `mode`; *taken: how many were.  Trajectories: from src through dst,
+// dst + hop, ... (elements).
 template <class E>
-cudaError_t march_t(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
+cudaError_t march_t(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t hop, int64_t nsteps, int64_t* taken)
 {
     constexpr bool f32 = std::is_same<E, float>::value;
-    const bool pull = c->cfg.pattern == MCLBM_PULL;
     const int vec = Q == 19 || !f32 ? 4 : 2;
     MarchArgs<E> a;
     memset(&a, 0, sizeof(a));
@@ -114,27 +115,32 @@ cudaError_t march_t(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
     const int64_t most = (kMaxUpdates / updates > 2 ? kMaxUpdates / updates : 2) & ~(int64_t)1;
     while (*taken < nsteps) {
         int64_t k = nsteps - *taken < most ? nsteps - *taken : most;
-        if (pull) k &= ~(int64_t)1;
+        if (mode == kMarchSwap) k &= ~(int64_t)1;
         if (k < 2 || !march_order(a, c, vec, k)) break;
         const size_t cnt_bytes = sizeof(int) * ((size_t)c->M << a.logU);
         if (cnt_bytes > kPartialBytes) break;
         a.cnt = (int*)(c->work + c->wl.partial);
         a.err = (int*)(c->work + c->wl.flag) + 1;
         fill_level<E>(a.lev, c);
-        a.lev.dst = (E*)lattice_ptr(c, pull ? c->cur : 0);
-        if (pull) a.lev.parity = 1;
+        if (mode == kMarchTrajectory) {
+            a.lev.src = *taken == 0 ? (const E*)src : (const E*)dst + (*taken - 1) * hop;
+            a.lev.dst = (E*)dst + *taken * hop;
+            a.hop = hop;
+        } else {
+            a.lev.dst = (E*)lattice_ptr(c, mode == kMarchSwap ? c->cur : 0);
+            if (mode == kMarchSwap) a.lev.parity = 1;
+        }
         cudaError_t e = cudaMemsetAsync(a.cnt, 0, cnt_bytes, c->stream);
         if (e != cudaSuccess) return e;
         if constexpr (f32)
-            e = launch_march_f32(a, pull, c->num_sms, tiles, c->stream);
+            e = launch_march_f32(a, mode, c->num_sms, tiles, c->stream);
         else
-            e = launch_march_f16(a, pull, c->num_sms, tiles, c->stream);
+            e = launch_march_f16(a, mode, c->num_sms, tiles, c->stream);
         if (e == cudaErrorCooperativeLaunchTooLarge) {  // part of the GPU only: launch by launch
             cudaGetLastError();
             break;
         }
         if (e != cudaSuccess) return e;
-        c->steps += k;
         *taken += k;
     }
     return cudaSuccess;
@@ -147,8 +153,24 @@ cudaError_t march_t(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
 cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
 {
     *taken = 0;
-    if (!march_serves(c, c->cfg.pattern == MCLBM_PULL ? nsteps & ~(int64_t)1 : nsteps)) return cudaSuccess;
-    return c->cfg.precision == MCLBM_FP32 ? march_t<float>(c, nsteps, taken) : march_t<__half>(c, nsteps, taken);
+    const int mode = c->cfg.pattern == MCLBM_PULL ? kMarchSwap : kMarchAA;
+    if (!march_serves(c, mode == kMarchSwap ? nsteps & ~(int64_t)1 : nsteps)) return cudaSuccess;
+    const cudaError_t e = c->cfg.precision == MCLBM_FP32 ? march_t<float>(c, mode, nullptr, nullptr, 0, nsteps, taken)
+                                                         : march_t<__half>(c, mode, nullptr, nullptr, 0, nsteps, taken);
+    c->steps += *taken;
+    return e;
+}
+
+// The same for pull steps from the lattice src through the lattices at dst, dst + hop_bytes, ..., each
+// of which keeps its state; the context's own state is not touched.
+cudaError_t launch_march_trajectory(mclbm_ctx* c, const void* src, void* dst, size_t hop_bytes, int64_t nsteps,
+                                    int64_t* taken)
+{
+    *taken = 0;
+    if (!march_serves(c, nsteps)) return cudaSuccess;
+    const int64_t hop = (int64_t)(hop_bytes / c->elem_bytes);
+    return c->cfg.precision == MCLBM_FP32 ? march_t<float>(c, kMarchTrajectory, src, dst, hop, nsteps, taken)
+                                          : march_t<__half>(c, kMarchTrajectory, src, dst, hop, nsteps, taken);
 }
 
 }  // namespace mclbm

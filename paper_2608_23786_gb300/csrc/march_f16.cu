@@ -3,9 +3,9 @@
 
 namespace mclbm {
 
-cudaError_t launch_march_f16(MarchArgs<__half>& a, bool pull, int num_sms, int64_t tiles, cudaStream_t s)
+cudaError_t launch_march_f16(MarchArgs<__half>& a, int mode, int num_sms, int64_t tiles, cudaStream_t s)
 {
-    return launch_march_vec<__half, 4>(a, pull, num_sms, tiles, s);
+    return launch_march_vec<__half, 4>(a, mode, num_sms, tiles, s);
 }
 
 }  // namespace mclbm

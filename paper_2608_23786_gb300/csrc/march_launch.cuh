@@ -5,11 +5,11 @@
 
 namespace mclbm {
 
-template <class E, int VEC, bool SWAP, bool WRAP>
+template <class E, int VEC, int MODE, bool WRAP>
 cudaError_t launch_march_variant(MarchArgs<E>& a, int num_sms, int64_t tiles, cudaStream_t s)
 {
     constexpr bool PACK = Storage<E>::shifted && VEC % 2 == 0;
-    auto kern = k_march<E, VEC, SWAP, PACK, WRAP>;
+    auto kern = k_march<E, VEC, MODE, PACK, WRAP>;
     // the register split of the kernel would wait forever with fewer registers at launch
     static std::atomic<int> regs_cache{0};
     int regs = regs_cache.load(std::memory_order_relaxed);
@@ -27,14 +27,20 @@ cudaError_t launch_march_variant(MarchArgs<E>& a, int num_sms, int64_t tiles, cu
 }
 
 template <class E, int VEC>
-cudaError_t launch_march_vec(MarchArgs<E>& a, bool pull, int num_sms, int64_t tiles, cudaStream_t s)
+cudaError_t launch_march_vec(MarchArgs<E>& a, int mode, int num_sms, int64_t tiles, cudaStream_t s)
 {
     const bool wrap = a.lev.g.N <= 32 * VEC;
-    if (pull)
-        return wrap ? launch_march_variant<E, VEC, true, true>(a, num_sms, tiles, s)
-                    : launch_march_variant<E, VEC, true, false>(a, num_sms, tiles, s);
-    return wrap ? launch_march_variant<E, VEC, false, true>(a, num_sms, tiles, s)
-                : launch_march_variant<E, VEC, false, false>(a, num_sms, tiles, s);
+    switch (mode) {
+        case kMarchAA:
+            return wrap ? launch_march_variant<E, VEC, kMarchAA, true>(a, num_sms, tiles, s)
+                        : launch_march_variant<E, VEC, kMarchAA, false>(a, num_sms, tiles, s);
+        case kMarchSwap:
+            return wrap ? launch_march_variant<E, VEC, kMarchSwap, true>(a, num_sms, tiles, s)
+                        : launch_march_variant<E, VEC, kMarchSwap, false>(a, num_sms, tiles, s);
+        default:
+            return wrap ? launch_march_variant<E, VEC, kMarchTrajectory, true>(a, num_sms, tiles, s)
+                        : launch_march_variant<E, VEC, kMarchTrajectory, false>(a, num_sms, tiles, s);
+    }
 }
 
 }  // namespace mclbm

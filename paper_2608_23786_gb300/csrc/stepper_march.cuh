@@ -22,6 +22,10 @@
 // the pull lattice two steps on, in place.  So pull contexts take an even number of steps here, in the
 // lattice that holds their state, and half the L2 that two lattices would need.
 //
+// Trajectories.  The adjoint keeps every state of a segment: there each step reads the pull lattice of the
+// state before and writes the next one's (kMarchTrajectory); what a step reads is still in L2, so
+// the states cross HBM once, outwards.
+//
 // Dependences.  cnt[sample][unit] counts the tiles finished, over all steps.  A tile at step a may
 // start when its unit and the two next to it have finished a * tiles_per_unit tiles: what it reads
 // is then written, and the slots it overwrites are no longer read.  The tile with the lowest position
@@ -56,9 +60,15 @@ static_assert(kMarchGroups * kMarchRegsWork + kMarchRegsBooks == (kMarchGroups +
 constexpr int kMarchAhead = 4;                   // tiles handed out beyond the last one reported
 constexpr uint64_t kMarchLimitNs = 1000ull * 1000 * 1000;  // 1 s of %globaltimer time per wait
 
+// What a step reads and writes: the AA pattern in place, the same with the slots of opposite velocities
+// exchanged (a pull lattice), or pull from one lattice to the next.
+enum MarchMode { kMarchAA = 0, kMarchSwap = 1, kMarchTrajectory = 2 };
+
 template <class E>
 struct MarchArgs {
-    LevelArgs<E> lev;  // dst: the lattice; parity: of the first step (pull lattices: 1)
+    LevelArgs<E> lev;  // dst: the lattice; parity: of the first step (pull lattices: 1).  Trajectories: src
+                       // the first state, dst the second
+    int64_t hop;       // trajectories: elements from a state's lattice to the next one's, from the second on
     unsigned steps;
     unsigned lanes, lag;
     unsigned logT;  // tiles per unit
@@ -169,6 +179,13 @@ __device__ __forceinline__ void st_release_cta(uint32_t p, int v)
     asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
 }
 
+// The lattice that step k reads (trajectories; k == steps: the last one written).
+template <class E>
+__device__ __forceinline__ E* march_state(const MarchArgs<E>& a, unsigned k)
+{
+    return k == 0 ? const_cast<E*>(a.lev.src) : a.lev.dst + (int64_t)(k - 1) * a.hop;
+}
+
 template <class E, int VEC>
 __device__ __forceinline__ RunLoc march_run(const MarchArgs<E>& a, const MarchTile& t)
 {
@@ -252,11 +269,12 @@ __device__ __forceinline__ void march_report(const MarchArgs<E>& a, MarchShared&
     }
 }
 
-// SWAP: the slots of opposite velocities are exchanged (a pull lattice).  WRAP: rows within one warp.
-template <class E, int VEC, bool SWAP, bool PACK, bool WRAP>
+// WRAP: rows within one warp.
+template <class E, int VEC, int MODE, bool PACK, bool WRAP>
 __global__ void __launch_bounds__(kMarchThreads, 1) k_march(const __grid_constant__ MarchArgs<E> a)
 {
     using C = typename Storage<E>::compute;
+    constexpr bool SWAP = MODE == kMarchSwap;
     __shared__ MarchShared sh;
     const int lane = threadIdx.x & 31;
     const Geom g = a.lev.g;
@@ -289,7 +307,9 @@ __global__ void __launch_bounds__(kMarchThreads, 1) k_march(const __grid_constan
         RunLoc p;
         if (have) {
             p = march_run<E, VEC>(a, cur);
-            if (p.mode == 1)
+            if constexpr (MODE == kMarchTrajectory)
+                finish_all<E, VEC, 0, WRAP>(g, p, lane, raw, v);
+            else if (p.mode == 1)
                 finish_all<E, VEC, 1, WRAP>(g, p, lane, raw, v);
             else
                 finish_all<E, VEC, 2, WRAP>(g, p, lane, raw, v);
@@ -312,16 +332,20 @@ __global__ void __launch_bounds__(kMarchThreads, 1) k_march(const __grid_constan
         }
         if (ok) {
             const RunLoc q = march_run<E, VEC>(a, nxt);
-            const E* src = a.lev.dst + (int64_t)q.m * Q * g.n;
-            if (q.mode == 1)
+            const E* src = (MODE == kMarchTrajectory ? march_state(a, nxt.step) : a.lev.dst) + (int64_t)q.m * Q * g.n;
+            if constexpr (MODE == kMarchTrajectory)
+                issue_all<E, VEC, 0, WRAP, true>(src, g, q, lane, raw);
+            else if (q.mode == 1)
                 issue_all<E, VEC, 1, WRAP, true, SWAP>(src, g, q, lane, raw);
             else
                 issue_all<E, VEC, 2, WRAP, true, SWAP>(src, g, q, lane, raw);
         }
         if (have) {
             collide_run<E, VEC, PACK>(v, a.lev);
-            E* base = a.lev.dst + (int64_t)p.m * Q * g.n;
-            if (p.mode == 1)
+            E* base = (MODE == kMarchTrajectory ? march_state(a, cur.step + 1) : a.lev.dst) + (int64_t)p.m * Q * g.n;
+            if constexpr (MODE == kMarchTrajectory)
+                scatter_all<E, VEC, 0>(base, g, p.x0, p.y, p.z, lane, v);
+            else if (p.mode == 1)
                 store_own_opp<E, VEC, SWAP>(base, g, p.node, v);
             else
                 scatter_all<E, VEC, 1, WRAP, SWAP>(base, g, p.x0, p.y, p.z, lane, v);
