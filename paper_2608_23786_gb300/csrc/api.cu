@@ -172,22 +172,21 @@ LaunchConfig default_launch(int precision, int pattern, int options)
 }
 
 // AA odd steps read and write shifted rows and favour other shapes (measured per parity at
-// 128^3 x 32 and 64^3 x 64): D3Q19 FP32 the two-stage cp.async ring with 4 nodes per thread,
-// FP16 the packed prefetching kernel with 4; D3Q27 FP32 and FP16 the packed prefetching kernel in
-// blocks of 256 (D3Q27 FP16 with the row rotation at 128^3: 83.2% of the copy bandwidth, against
-// 80.7% for the ring and 52% for the one-node prefetching kernel without the rotation).
-// Nmax: the largest lattice the shape serves (a context's N, a batch's largest level): D3Q19 FP16
-// odd steps with Nmax <= 256 take the two-stage ring with 8 nodes per thread, whose rows of up to
-// 256 nodes lie within one warp and rotate (128^3 x 32: 81.4% of the copy bandwidth against 80.7%
-// for the packed prefetching kernel with 4; the three-level batch 64^3 x 64 + 128^3 x 32 + 256^3 x 8:
-// 84.2% per macro step against 77.7% with rows of 256 nodes spanning warps).
+// 128^3 x 32 and 64^3 x 64): D3Q19 FP32 the three-slot cp.async ring with 4 nodes per thread, FP16 the
+// two-slot kind with 8 where a row of up to 256 nodes lies within one warp (one slot refilled as it is
+// read: 128^3 x 32 80.3 GLUPS against 74.4 with two slots and 70 for the packed prefetching kernel with
+// 4) and the packed prefetching kernel with 4 beyond (512^3 60.5; the ring 66.3); D3Q27 FP32 and FP16 the packed prefetching kernel in blocks of 256 (D3Q27 FP16
+// with the row rotation at 128^3: 83.2% of the copy bandwidth, against 80.7% for the ring and 52% for
+// the one-node prefetching kernel without the rotation).
+// Nmax: the largest lattice the shape serves (a context's N, a batch's largest level).  D3Q27 FP16 rows
+// of more than 128 nodes span warps, where the ring measured 39.6 GLUPS against 21.4 at 256^3.
 LaunchConfig default_launch_odd(int precision, int pattern, int options, int Nmax)
 {
     const LaunchConfig even = default_launch(precision, pattern, options);
     if (pattern != MCLBM_AA || even.kind == 6 || precision == MCLBM_FP64) return even;
 #ifdef MCLBM_D3Q27
-    (void)Nmax;
-    return precision == MCLBM_FP32 ? LaunchConfig{2, 256, 3} : LaunchConfig{4, 256, 3};
+    if (precision == MCLBM_FP32) return LaunchConfig{2, 256, 3};
+    return Nmax <= 32 * 4 ? LaunchConfig{4, 256, 3} : LaunchConfig{4, 128, 4};
 #else
     if (precision == MCLBM_FP32) return LaunchConfig{4, 128, 5};
     if (Nmax <= 32 * 8) return LaunchConfig{8, 128, 4};

@@ -206,4 +206,58 @@ __global__ void __launch_bounds__(BLOCK) k_step_async(const BatchArgs<E> args)
     cp_async_wait<0>();  // nothing may stay in flight into a buffer that is released at exit
 }
 
+// The ring with a single slot: a thread reads its run from the slot, refills the slot with its next
+// run, and collides and stores the run it holds while the copies land.  The same distance ahead as two
+// slots with half the shared memory.
+template <class E, int VEC, int PATTERN, int BLOCK, int FIX, bool WRAP = false, bool ONE = false>
+__global__ void __launch_bounds__(BLOCK) k_step_slot(const BatchArgs<E> args)
+{
+    static_assert(Storage<E>::shifted, "the shared-memory prefetch variant serves the FP32 and FP16 storage");
+    static_assert(sizeof(E) == 4 || VEC % 2 == 0, "FP16 runs must be whole 4-byte words");
+    using C = typename Storage<E>::compute;
+    using Ring = AsyncRing<E, VEC, BLOCK, 1>;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    const int64_t total = args.prefix[args.nlev];
+    const int64_t stride = (int64_t)gridDim.x * BLOCK;
+    int64_t t = blockIdx.x * (int64_t)BLOCK + threadIdx.x;
+    if (t >= total) return;  // whole warps: totals and strides are multiples of 32
+    Ring ring;
+    ring.base = (uint32_t)__cvta_generic_to_shared(smem);
+    ring.tid = threadIdx.x;
+    RunLoc cur = locate<E, VEC, ONE>(args, t, PATTERN);
+    {
+        const LevelArgs<E>& L = args.lev[ONE ? 0 : cur.l];
+        async_issue_all<E, VEC, BLOCK, 1, FIX, WRAP>(L.src + (int64_t)cur.m * Q * L.g.n, L.g, cur, lane, ring, 0);
+    }
+    for (;;) {
+        cp_async_commit();
+        cp_async_wait<0>();
+        const LevelArgs<E>& L = args.lev[ONE ? 0 : cur.l];
+        const Geom g = L.g;
+        C v[Q][VEC];
+        async_finish_all<E, VEC, BLOCK, 1, FIX, WRAP>(smem, 0, threadIdx.x, g, cur, lane, v);
+        __syncwarp();  // the slot is read before it is refilled
+        t += stride;
+        const bool more = t < total;
+        RunLoc nxt = cur;
+        if (more) {
+            nxt = locate<E, VEC, ONE>(args, t, PATTERN);
+            const LevelArgs<E>& Ln = args.lev[ONE ? 0 : nxt.l];
+            async_issue_all<E, VEC, BLOCK, 1, FIX, WRAP>(Ln.src + (int64_t)nxt.m * Q * Ln.g.n, Ln.g, nxt, lane, ring, 0);
+        }
+        collide_run<E, VEC, (VEC % 2 == 0)>(v, L);
+        E* base = L.dst + (int64_t)cur.m * Q * g.n;
+        const int mode = FIX >= 0 ? FIX : cur.mode;
+        if (mode == 0)
+            scatter_all<E, VEC, 0>(base, g, cur.x0, cur.y, cur.z, lane, v);
+        else if (mode == 1)
+            store_own_opp<E, VEC>(base, g, cur.node, v);
+        else
+            scatter_all<E, VEC, 1, WRAP>(base, g, cur.x0, cur.y, cur.z, lane, v);
+        if (!more) break;
+        cur = nxt;
+    }
+}
+
 }  // namespace mclbm

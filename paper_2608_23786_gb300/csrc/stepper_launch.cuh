@@ -96,8 +96,16 @@ cudaError_t launch_prefetch_variant(const BatchArgs<E>& a, int grid_cap, cudaStr
 template <class E, int VEC, int PATTERN, int BLOCK, int FIX, int STAGES, bool WRAP, bool ONE>
 cudaError_t launch_async_fixed(const BatchArgs<E>& a, int grid_cap, cudaStream_t s, int* occupancy_out)
 {
-    auto kern = k_step_async<E, VEC, PATTERN, BLOCK, FIX, STAGES, WRAP, ONE>;
-    constexpr int smem = AsyncRing<E, VEC, BLOCK, STAGES>::kBytes;
+    const auto pick = [] {
+        if constexpr (STAGES == 1)
+            return k_step_slot<E, VEC, PATTERN, BLOCK, FIX, WRAP, ONE>;
+        else
+            return k_step_async<E, VEC, PATTERN, BLOCK, FIX, STAGES, WRAP, ONE>;
+    };
+    auto kern = pick();
+    // rows that rotate and own rows have no edge words
+    constexpr int smem = WRAP || FIX == 1 ? AsyncRing<E, VEC, BLOCK, STAGES>::kVecBytes
+                                          : AsyncRing<E, VEC, BLOCK, STAGES>::kBytes;
     static std::atomic<int> occ_cache[kMaxDevices];
     int occ = 0;
     const cudaError_t e = resident_blocks(kern, BLOCK, smem, occ_cache, &occ);
@@ -122,17 +130,22 @@ cudaError_t launch_async_levels(const BatchArgs<E>& a, int grid_cap, cudaStream_
     // bound, loses with it: AA odd 100% -> 89%, so FP32 ring launches keep the end elements)
     constexpr bool kWrapKind = std::is_same<E, __half>::value;
     const bool wrap = kWrapKind && rows_in_warp(a, VEC);
+    // two slots (kind 4), FP16, shifted loads: one slot refilled as soon as it is read (k_step_slot;
+    // measured at 128^3 x 32: D3Q19 AA odd steps 74.4 -> 80.3 GLUPS, pull 83.4 -> 84.4, 512^3 pull 75.1 ->
+    // 78.9; D3Q27 pull 52.5 -> 53.3, but 48.0 -> 46.6 where rows span warps).  AA even steps lose with it
+    // (80.4 -> 70.5) and keep two.
+    constexpr int kShifted = std::is_same<E, __half>::value && STAGES == 2 ? 1 : STAGES;
     if constexpr (PATTERN == 0) {
         if constexpr (kWrapKind)
-            if (wrap) return launch_async_fixed<E, VEC, 0, BLOCK, 0, STAGES, true, ONE>(a, grid_cap, s, occ);
-        return launch_async_fixed<E, VEC, 0, BLOCK, 0, STAGES, false, ONE>(a, grid_cap, s, occ);
+            if (wrap) return launch_async_fixed<E, VEC, 0, BLOCK, 0, kShifted, true, ONE>(a, grid_cap, s, occ);
+        return launch_async_fixed<E, VEC, 0, BLOCK, 0, Q == 19 ? kShifted : STAGES, false, ONE>(a, grid_cap, s, occ);
     } else {
         const int par = launch_parity(a);
         if (par == 0) return launch_async_fixed<E, VEC, 1, BLOCK, 1, STAGES, false, ONE>(a, grid_cap, s, occ);
         if (par == 1) {
             if constexpr (kWrapKind)
-                if (wrap) return launch_async_fixed<E, VEC, 1, BLOCK, 2, STAGES, true, ONE>(a, grid_cap, s, occ);
-            return launch_async_fixed<E, VEC, 1, BLOCK, 2, STAGES, false, ONE>(a, grid_cap, s, occ);
+                if (wrap) return launch_async_fixed<E, VEC, 1, BLOCK, 2, kShifted, true, ONE>(a, grid_cap, s, occ);
+            return launch_async_fixed<E, VEC, 1, BLOCK, 2, Q == 19 ? kShifted : STAGES, false, ONE>(a, grid_cap, s, occ);
         }
         return cudaErrorInvalidValue;
     }
