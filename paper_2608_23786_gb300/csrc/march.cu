@@ -7,8 +7,8 @@
 
 namespace mclbm {
 
-cudaError_t launch_march_f32(MarchArgs<float>& a, int mode, int num_sms, int64_t tiles, cudaStream_t s);
-cudaError_t launch_march_f16(MarchArgs<__half>& a, int mode, int num_sms, int64_t tiles, cudaStream_t s);
+cudaError_t launch_march_f32(MarchArgs<float>& a, int vec, int mode, int num_sms, int64_t tiles, cudaStream_t s);
+cudaError_t launch_march_f16(MarchArgs<__half>& a, int vec, int mode, int num_sms, int64_t tiles, cudaStream_t s);
 
 namespace {
 
@@ -84,14 +84,14 @@ bool march_order(MarchArgs<E>& a, const mclbm_ctx* c, int vec, int64_t steps)
 // The kernel's start (counters, cooperative launch, fill and drain) costs about 11 us a call.
 //
 // FP32 storage, whose launch per step is at the HBM bound: per step the kernel saves 1 to 2 us below
-// 2^16 nodes (4.2 against 3.5 us at 8^3 to 32^3), 3 us at 32^3 x 7 (8.3 against 5.4), 4 us at 64^3 (10.4
-// against 6.4), and a third of the time from 64^3 x 2 on (64^3 x 64 381 against 273 us, AA 387 against
-// 261; 128^3 x 8 385 against 273).  Three steps: 64^3 x 2 AA 47.9 against 38.9 us, 64^3 34.1 against 30.9
+// 2^16 nodes (4.2 against 2.6 to 3.8 us at 8^3 to 32^3), 3 us at 32^3 x 7 (8.3 against 5.0), 4 us at 64^3
+// (10.4 against 5.9), and a third of the time from 64^3 x 2 on (64^3 x 64 381 against 271 us, AA 387 against
+// 261; 128^3 x 8 385 against 270).  Three steps: 64^3 x 2 AA 47.9 against 38.9 us, 64^3 34.1 against 30.9
 // us, 32^3 x 3 23.3 against 25.1 us.
 //
 // FP16 storage is bound by arithmetic, in a kernel with twice the nodes per thread (65 against 78 GLUPS
-// at 64^3 x 64): here only what is bound by launches and latency, 6.2 against 3.1 to 3.5 us per step up
-// to 32^3, 64^3 8.3 against 5.3, 64^3 x 4 18.5 against 16.4 (D3Q27 64^3 x 2 14.4 against 13.7 us).
+// at 64^3 x 64): here only what is bound by launches and latency, 6.2 against 2.4 to 3.5 us per step up
+// to 32^3, 64^3 8.3 against 5.2, 64^3 x 4 18.5 against 16.4 (D3Q27 64^3 x 2 14.4 against 13.2 us).
 // FP64 storage is bound by its arithmetic from 32^3 on.
 bool march_serves(const mclbm_ctx* c, int64_t steps)
 {
@@ -101,13 +101,24 @@ bool march_serves(const mclbm_ctx* c, int64_t steps)
     return steps >= (nodes < (1 << 16) ? 12 : (nodes < (1 << 18) ? 6 : 3));
 }
 
+// Nodes per thread.  Four keep more independent work per warp, two halve a tile's latency and spread
+// a small ensemble over more warps.  FP32: two up to 64^3 nodes (8^3 3.4 -> 2.6 us per step, 32^3 3.9 ->
+// 3.1, 32^3 x 7 5.4 -> 5.0, 64^3 6.3 -> 5.9, but 64^3 x 2 8.9 -> 10.8; D3Q27 32^3 4.9 -> 3.4, 64^3 8.5 ->
+// 7.2, 64^3 x 2 12.9 -> 13.9).  FP16: two up to 32^3 x 4 (32^3 3.4 -> 3.0, 32^3 x 7 4.5 -> 4.7), D3Q27, whose
+// four and the four ahead spill, always (64^3 x 2 13.5 -> 13.2).  D3Q27 FP32 rows that span warps: two.
+int march_vec(int precision, int N, int64_t nodes)
+{
+    if (Q == 27) return precision == MCLBM_FP16 || nodes <= (1 << 18) || N > 128 ? 2 : 4;
+    return nodes <= (precision == MCLBM_FP32 ? 1 << 18 : 1 << 17) ? 2 : 4;
+}
+
 // Takes `nsteps` steps in mode `mode`; *taken: how many were.  Trajectories: from src through dst,
 // dst + hop, ... (elements).
 template <class E>
 cudaError_t march_t(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t hop, int64_t nsteps, int64_t* taken)
 {
     constexpr bool f32 = std::is_same<E, float>::value;
-    const int vec = Q == 19 || !f32 ? 4 : 2;
+    const int vec = march_vec(c->cfg.precision, c->N, (int64_t)c->M * c->n);
     MarchArgs<E> a;
     memset(&a, 0, sizeof(a));
     const int64_t tiles = (int64_t)c->M * c->n / (kMarchGroup * vec);
@@ -133,9 +144,9 @@ cudaError_t march_t(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t 
         cudaError_t e = cudaMemsetAsync(a.cnt, 0, cnt_bytes, c->stream);
         if (e != cudaSuccess) return e;
         if constexpr (f32)
-            e = launch_march_f32(a, mode, c->num_sms, tiles, c->stream);
+            e = launch_march_f32(a, vec, mode, c->num_sms, tiles, c->stream);
         else
-            e = launch_march_f16(a, mode, c->num_sms, tiles, c->stream);
+            e = launch_march_f16(a, vec, mode, c->num_sms, tiles, c->stream);
         if (e == cudaErrorCooperativeLaunchTooLarge) {  // part of the GPU only: launch by launch
             cudaGetLastError();
             break;

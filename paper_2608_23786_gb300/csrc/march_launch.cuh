@@ -22,24 +22,22 @@ cudaError_t launch_march_variant(MarchArgs<E>& a, int num_sms, int64_t tiles, cu
     if (regs != kMarchRegs) return cudaErrorInvalidConfiguration;
     // one block per SM (its registers fill it); a small ensemble takes a block per tile
     const int64_t grid = num_sms < tiles ? num_sms : tiles;
+    constexpr int smem = march_smem<E, VEC, kMarchSlot<E, VEC, WRAP>>();
+    if constexpr (smem > 0) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
     void* args[] = {&a};
-    return cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(kMarchThreads), args, 0, s);
+    return cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(kMarchThreads), args, smem, s);
 }
 
-template <class E, int VEC>
-cudaError_t launch_march_vec(MarchArgs<E>& a, int mode, int num_sms, int64_t tiles, cudaStream_t s)
+template <class E, int VEC, bool WRAP>
+cudaError_t launch_march_mode(MarchArgs<E>& a, int mode, int num_sms, int64_t tiles, cudaStream_t s)
 {
-    const bool wrap = a.lev.g.N <= 32 * VEC;
     switch (mode) {
-        case kMarchAA:
-            return wrap ? launch_march_variant<E, VEC, kMarchAA, true>(a, num_sms, tiles, s)
-                        : launch_march_variant<E, VEC, kMarchAA, false>(a, num_sms, tiles, s);
-        case kMarchSwap:
-            return wrap ? launch_march_variant<E, VEC, kMarchSwap, true>(a, num_sms, tiles, s)
-                        : launch_march_variant<E, VEC, kMarchSwap, false>(a, num_sms, tiles, s);
-        default:
-            return wrap ? launch_march_variant<E, VEC, kMarchTrajectory, true>(a, num_sms, tiles, s)
-                        : launch_march_variant<E, VEC, kMarchTrajectory, false>(a, num_sms, tiles, s);
+        case kMarchAA: return launch_march_variant<E, VEC, kMarchAA, WRAP>(a, num_sms, tiles, s);
+        case kMarchSwap: return launch_march_variant<E, VEC, kMarchSwap, WRAP>(a, num_sms, tiles, s);
+        default: return launch_march_variant<E, VEC, kMarchTrajectory, WRAP>(a, num_sms, tiles, s);
     }
 }
 

@@ -64,14 +64,15 @@ __device__ __forceinline__ const void* edge_word(const E* row, int e)
 }
 
 // WRAP: every row lies within one warp and its lanes rotate (row_lane), so no edge word is copied.
-template <class E, int VEC, int BLOCK, int STAGES, int FIX, bool WRAP = false, int I = 0>
+// SWAP: the slots of opposite velocities are exchanged (stepper_march.cuh).
+template <class E, int VEC, int BLOCK, int STAGES, int FIX, bool WRAP = false, bool SWAP = false, int I = 0>
 __device__ __forceinline__ void async_issue_all(const E* base, const Geom& g, const RunLoc& p, int lane,
                                                 const AsyncRing<E, VEC, BLOCK, STAGES>& ring, int stage)
 {
     if constexpr (I < Q) {
         const int mode = FIX >= 0 ? FIX : p.mode;
         const bool shift = mode != 1;
-        const int slot = mode == 2 ? Dir<I>::o : I;
+        const int slot = (mode == 2) != SWAP ? Dir<I>::o : I;
         const int ry = shift ? g.wrap(p.y - Dir<I>::y) : p.y;
         const int rz = shift ? g.wrap(p.z - Dir<I>::z) : p.z;
         const E* row = base + (int64_t)slot * g.n + g.node(0, ry, rz);
@@ -84,7 +85,7 @@ __device__ __forceinline__ void async_issue_all(const E* base, const Geom& g, co
             if (shift && (lane == 31 || p.x0 + VEC == g.N))
                 cp_async<4>(ring.edge_slot(stage, I), edge_word(row, (p.x0 + VEC) & (g.N - 1)));
         }
-        async_issue_all<E, VEC, BLOCK, STAGES, FIX, WRAP, I + 1>(base, g, p, lane, ring, stage);
+        async_issue_all<E, VEC, BLOCK, STAGES, FIX, WRAP, SWAP, I + 1>(base, g, p, lane, ring, stage);
     }
 }
 

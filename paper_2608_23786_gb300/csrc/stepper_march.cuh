@@ -43,6 +43,7 @@
 // when that tile has been handed out; otherwise it finishes its current tile first.  What other
 // blocks stored is read with coherent loads (ld_cg).
 #pragma once
+#include "stepper_async.cuh"
 #include "stepper_impl.cuh"
 #include "stepper_staged.cuh"
 
@@ -58,6 +59,9 @@ constexpr int kMarchRegs = 168, kMarchRegsWork = 240, kMarchRegsBooks = 24;
 static_assert(kMarchGroups * kMarchRegsWork + kMarchRegsBooks == (kMarchGroups + 1) * kMarchRegs,
               "a split takes no more registers than the launch has");
 constexpr int kMarchAhead = 4;                   // tiles handed out beyond the last one reported
+// Pause between two looks of the warps that keep the books: without it they take issue slots from the
+// colliding warps of their partition (pull 64^3 x 64 61.5 -> 62.1 GLUPS, in another build 59.0 -> 62.1).
+constexpr unsigned kMarchNapNs = 64;
 constexpr uint64_t kMarchLimitNs = 1000ull * 1000 * 1000;  // 1 s of %globaltimer time per wait
 
 // What a step reads and writes: the AA pattern in place, the same with the slots of opposite velocities
@@ -239,6 +243,7 @@ __device__ __forceinline__ void march_hand_out(const MarchArgs<E>& a, MarchShare
             bool go = room;
             if (go && t.valid && lane < 3) go = ld_acquire_gpu(c) >= need;
             if (__all_sync(0xffffffffu, go)) break;
+            __nanosleep(kMarchNapNs);
             if ((it & 63) == 0 && __any_sync(0xffffffffu, lane == 0 && march_give_up(t0, a.err))) return;
         }
         if (lane == 0) {
@@ -259,6 +264,7 @@ __device__ __forceinline__ void march_report(const MarchArgs<E>& a, MarchShared&
     for (int n = 0;; ++n) {
         const uint64_t t0 = global_ns();
         for (unsigned it = 1; !mbar_test(bar + 8 * (n & (kMarchAhead - 1)), (n / kMarchAhead) & 1); ++it) {
+            __nanosleep(kMarchNapNs);
             if ((it & 15) == 0 && ld_acquire_cta(smem_u32(&sh.last[g])) == n) return;
             if ((it & 255) == 0 && march_give_up(t0, a.err)) return;
         }
@@ -269,12 +275,27 @@ __device__ __forceinline__ void march_report(const MarchArgs<E>& a, MarchShared&
     }
 }
 
+// Whether the run ahead waits in shared memory (one cp.async slot a thread, as in k_step_slot) instead of
+// registers: D3Q27 FP32, whose run of four nodes and the one ahead do not fit the registers together
+// (16-byte copies, which go through L2 only, and no edge words): 64^3 x 16 109 -> 99 us per step against two
+// nodes per thread in registers, AA 105 -> 99.
+template <class E, int VEC, bool WRAP>
+constexpr bool kMarchSlot = Q == 27 && WRAP && sizeof(E) == 4 && VEC == 4;
+
+template <class E, int VEC, bool SLOT>
+constexpr int march_smem()
+{
+    return SLOT ? AsyncRing<E, VEC, kMarchGroups * kMarchGroup, 1>::kVecBytes : 0;
+}
+
 // WRAP: rows within one warp.
 template <class E, int VEC, int MODE, bool PACK, bool WRAP>
 __global__ void __launch_bounds__(kMarchThreads, 1) k_march(const __grid_constant__ MarchArgs<E> a)
 {
     using C = typename Storage<E>::compute;
-    constexpr bool SWAP = MODE == kMarchSwap;
+    constexpr bool SWAP = MODE == kMarchSwap, SLOT = kMarchSlot<E, VEC, WRAP>;
+    constexpr int kRing = kMarchGroups * kMarchGroup;
+    extern __shared__ __align__(16) unsigned char march_dyn[];
     __shared__ MarchShared sh;
     const int lane = threadIdx.x & 31;
     const Geom g = a.lev.g;
@@ -301,13 +322,25 @@ __global__ void __launch_bounds__(kMarchThreads, 1) k_march(const __grid_constan
     bool have = false;  // cur is loaded
     bool ended = false;
     int j = -1;  // number of cur among the group's tiles (of the last one when !have)
-    RawRun<E, VEC> raw[Q];
+    RawRun<E, VEC> raw[SLOT ? 1 : Q];
+    AsyncRing<E, VEC, kRing, 1> ring;
+    ring.base = SLOT ? smem_u32(march_dyn) : 0u;
+    ring.tid = threadIdx.x;
     for (;;) {
         C v[Q][VEC];
         RunLoc p;
         if (have) {
             p = march_run<E, VEC>(a, cur);
-            if constexpr (MODE == kMarchTrajectory)
+            if constexpr (SLOT) {
+                cp_async_wait<0>();
+                if constexpr (MODE == kMarchTrajectory)
+                    async_finish_all<E, VEC, kRing, 1, 0, WRAP>(march_dyn, 0, threadIdx.x, g, p, lane, v);
+                else if (p.mode == 1)
+                    async_finish_all<E, VEC, kRing, 1, 1, WRAP>(march_dyn, 0, threadIdx.x, g, p, lane, v);
+                else
+                    async_finish_all<E, VEC, kRing, 1, 2, WRAP>(march_dyn, 0, threadIdx.x, g, p, lane, v);
+                __syncwarp();  // the slot is read before it is refilled
+            } else if constexpr (MODE == kMarchTrajectory)
                 finish_all<E, VEC, 0, WRAP>(g, p, lane, raw, v);
             else if (p.mode == 1)
                 finish_all<E, VEC, 1, WRAP>(g, p, lane, raw, v);
@@ -333,7 +366,15 @@ __global__ void __launch_bounds__(kMarchThreads, 1) k_march(const __grid_constan
         if (ok) {
             const RunLoc q = march_run<E, VEC>(a, nxt);
             const E* src = (MODE == kMarchTrajectory ? march_state(a, nxt.step) : a.lev.dst) + (int64_t)q.m * Q * g.n;
-            if constexpr (MODE == kMarchTrajectory)
+            if constexpr (SLOT) {  // cp.async.cg: through L2, as ld_cg
+                if constexpr (MODE == kMarchTrajectory)
+                    async_issue_all<E, VEC, kRing, 1, 0, WRAP>(src, g, q, lane, ring, 0);
+                else if (q.mode == 1)
+                    async_issue_all<E, VEC, kRing, 1, 1, WRAP, SWAP>(src, g, q, lane, ring, 0);
+                else
+                    async_issue_all<E, VEC, kRing, 1, 2, WRAP, SWAP>(src, g, q, lane, ring, 0);
+                cp_async_commit();
+            } else if constexpr (MODE == kMarchTrajectory)
                 issue_all<E, VEC, 0, WRAP, true>(src, g, q, lane, raw);
             else if (q.mode == 1)
                 issue_all<E, VEC, 1, WRAP, true, SWAP>(src, g, q, lane, raw);

@@ -28,8 +28,8 @@ def _same(a, b):
 
 @pytest.mark.parametrize("lattice", [19, 27])
 @pytest.mark.parametrize("pattern", ["pull", "aa"])
-@pytest.mark.parametrize("N,M,steps", [(8, 1, 12), (8, 131, 12), (16, 3, 13), (32, 7, 17), (64, 1, 6), (64, 9, 23),
-                                       (128, 2, 7), (256, 1, 5)])
+@pytest.mark.parametrize("N,M,steps", [(8, 1, 12), (8, 131, 12), (8, 600, 5), (16, 3, 13), (32, 7, 17),
+                                       (32, 12, 5), (64, 1, 6), (64, 9, 23), (128, 2, 7), (256, 1, 5)])
 def test_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
     a, b = _pair(N, M, pattern=pattern, lattice=lattice)
     a.step(steps)
@@ -40,7 +40,7 @@ def test_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
 
 @pytest.mark.parametrize("lattice", [19, 27])
 @pytest.mark.parametrize("pattern", ["pull", "aa"])
-@pytest.mark.parametrize("N,M,steps", [(8, 1, 7), (16, 3, 6), (32, 7, 9), (64, 2, 6)])
+@pytest.mark.parametrize("N,M,steps", [(8, 1, 7), (16, 3, 6), (32, 4, 8), (32, 7, 9), (64, 2, 6)])
 def test_fp16_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
     a, b = _pair(N, M, "fp16", pattern=pattern, lattice=lattice)
     a.step(steps)
