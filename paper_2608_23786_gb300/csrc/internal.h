@@ -108,7 +108,8 @@ void* lattice_ptr(const mclbm_ctx* c, int which);
 // kernels (launchers return cudaError_t of the launch)
 cudaError_t launch_init(const mclbm_ctx* c, const double* d_params);
 cudaError_t launch_step(mclbm_ctx* c);  // one step of one context; updates cur and steps
-cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken);  // march.cu
+bool march_serves_call(const mclbm_ctx* c, int64_t nsteps);                 // march.cu
+cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken);
 cudaError_t launch_march_trajectory(mclbm_ctx* c, const void* src, void* dst, size_t hop_bytes, int64_t nsteps,
                                     int64_t* taken);
 cudaError_t launch_step_with(mclbm_ctx* c, const LaunchConfig& cfg, const LaunchConfig& cfg_odd);

@@ -159,13 +159,18 @@ cudaError_t march_t(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t 
 
 }  // namespace
 
+bool march_serves_call(const mclbm_ctx* c, int64_t nsteps)
+{
+    return march_serves(c, c->cfg.pattern == MCLBM_PULL ? nsteps & ~(int64_t)1 : nsteps);
+}
+
 // Takes steps of a call for `nsteps` steps in the multi-step kernel, where it serves the context;
 // *taken is the number taken (the caller takes the others launch by launch).
 cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
 {
     *taken = 0;
     const int mode = c->cfg.pattern == MCLBM_PULL ? kMarchSwap : kMarchAA;
-    if (!march_serves(c, mode == kMarchSwap ? nsteps & ~(int64_t)1 : nsteps)) return cudaSuccess;
+    if (!march_serves_call(c, nsteps)) return cudaSuccess;
     const cudaError_t e = c->cfg.precision == MCLBM_FP32 ? march_t<float>(c, mode, nullptr, nullptr, 0, nsteps, taken)
                                                          : march_t<__half>(c, mode, nullptr, nullptr, 0, nsteps, taken);
     c->steps += *taken;

@@ -63,3 +63,21 @@ def test_a_chosen_shape_keeps_a_launch_per_step():
     a, b = _pair(32, 20)
     mclbm.mclbm_set_launch(b.ctx, 1, 128, 0)
     _same(a.step(14), b.step(14))
+
+
+@pytest.mark.parametrize("precision,macro", [("fp32", 1), ("fp32", 3), ("fp16", 6)])
+@pytest.mark.parametrize("pattern", ["pull", "aa"])
+def test_batch_level_by_level_equals_single_steps(precision, macro, pattern):
+    """Levels that the multi-step kernel serves, and one (the coarsest, a few steps) that it does not."""
+    pairs = [_pair(16 << k, M, precision, pattern=pattern) for k, M in enumerate((6, 3, 2))]
+    b = mclbm.mclbm_batch_create([a.ctx for a, _ in pairs], [1, 4, 16])
+    try:
+        mclbm.mclbm_batch_step(b, macro)
+        mclbm.mclbm_batch_step(b, 1)
+        assert mclbm.mclbm_batch_macro_steps(b) == macro + 1
+        for (x, y), sub in zip(pairs, (1, 4, 16)):
+            for _ in range(sub * (macro + 1)):
+                y.step(1)
+            _same(x, y)
+    finally:
+        mclbm.mclbm_batch_destroy(b)
