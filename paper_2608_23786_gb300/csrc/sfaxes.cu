@@ -21,7 +21,11 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kMaxP = 8;
-constexpr int kSfBlocks = 152 * 2;
+
+// Blocks over the 3 N^2 lines, whose loads' latency more blocks per SM hide: 2, 4, 6, 8 per SM take 1175,
+// 1080, 1053, 1049 us at N = 128 x 4 and 3.29, 3.09, 2.99, 2.95 ms at 256^3 (FP32).  Below N = 64, where
+// there are few lines, the partial sums of more blocks would need more scratch than the spectrum's.
+int sf_blocks(int N) { return 152 * (N < 64 ? 2 : 6); }
 
 __global__ void __launch_bounds__(kThreads) k_sf_axes(const double* __restrict__ u, int N, int logN, int pmax,
                                                       double* __restrict__ partial)
@@ -224,7 +228,7 @@ size_t sf_axes_smem(int N)
     return a > b ? a : b;
 }
 
-size_t sf_axes_partial_bytes(int N) { return (size_t)kSfBlocks * (N / 2) * (kMaxP - 1) * sizeof(double); }
+size_t sf_axes_partial_bytes(int N) { return (size_t)sf_blocks(N) * (N / 2) * (kMaxP - 1) * sizeof(double); }
 
 cudaError_t launch_sf_axes(mclbm_ctx* c, int pmax, double* h_S)
 {
@@ -242,10 +246,10 @@ cudaError_t launch_sf_axes(mclbm_ctx* c, int pmax, double* h_S)
     for (int m = 0; m < c->M; ++m) {
         if ((e = launch_field(c, m, field)) != cudaSuccess) return e;
         if (f32)
-            k_sf_axes_f32<<<kSfBlocks, kThreads, smem, c->stream>>>(field, N, c->logN, partial);
+            k_sf_axes_f32<<<sf_blocks(N), kThreads, smem, c->stream>>>(field, N, c->logN, partial);
         else
-            k_sf_axes<<<kSfBlocks, kThreads, smem, c->stream>>>(field, N, c->logN, pmax, partial);
-        k_sf_reduce<<<(halfN * (pmax - 1) + 7) / 8, 256, 0, c->stream>>>(partial, kSfBlocks, halfN, pmax, scale,
+            k_sf_axes<<<sf_blocks(N), kThreads, smem, c->stream>>>(field, N, c->logN, pmax, partial);
+        k_sf_reduce<<<(halfN * (pmax - 1) + 7) / 8, 256, 0, c->stream>>>(partial, sf_blocks(N), halfN, pmax, scale,
                                                out + (int64_t)m * (pmax - 1) * halfN);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
