@@ -1,14 +1,15 @@
 """Benchmark of the Monte Carlo KBC LBM hot path on one GB300 (or N, one ensemble per rank).
 
 Workload (default): M = 64 randomized Taylor-Green samples on 64^3, Re = 800, Ma = 0.025,
-shifted FP32 populations, pull streaming; the whole ensemble advances in one launch per
-lattice step.  One bench step = one output interval: S = 50 fused stream+collide updates
+shifted FP32 populations, pull streaming; the ensemble's updates of a call run in one launch of
+the multi-step kernel.  One bench step = one output interval: S = 50 fused stream+collide updates
 of every sample, then the ensemble reductions the interval feeds (per-sample kinetic
 energy E_m(t), ensemble mean and variance velocity fields, all FP64).
 
 metric: ensemble GLUPS (lattice-node updates per second, summed over ranks), with the
-stepper's achieved HBM bandwidth against the measured copy bandwidth.  Inputs (one
-ensemble of 2.55 GB of populations) exceed the 129 MB L2, so no flush is needed.
+bytes per second that the stepper's updates read and write: against the measured copy bandwidth of
+HBM where a step is a launch, against the copy rate within L2 for the multi-step kernel.  Inputs (one
+ensemble of 1.27 GB of populations) exceed the 129 MB L2, so no flush is needed.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 """
@@ -32,12 +33,18 @@ KINDS = ["direct", "staged", "prefetch", "prefetch_packed", "async_ring2", "asyn
 KERNEL_NAMES = ["k_step_batch", "k_step_staged", "k_step_prefetch", "k_step_prefetch", "k_step_async", "k_step_async",
                 "k_step_batch"]
 BYTES_PER_LU = {"fp64": 2 * 19 * 8, "fp32": 2 * 19 * 4, "fp16": 2 * 19 * 2}
+# The multi-step kernel (several updates of an ensemble per launch, inputs found in L2) and what its
+# accesses are set against: a copy of 64^3 FP32 lattices within L2, measured at 12.7 to 13.4 TB/s.
+MULTI_STEP_KERNEL = "k_march"
+L2_COPY_GBS = 12700.0
 STEPPER_SOURCES = ["paper_2608_23786_gb300/csrc/stepper.cu", "paper_2608_23786_gb300/csrc/collide.cuh",
                    "paper_2608_23786_gb300/csrc/storage.cuh", "paper_2608_23786_gb300/csrc/lattice.cuh",
                    "paper_2608_23786_gb300/csrc/stepper_impl.cuh", "paper_2608_23786_gb300/csrc/stepper_launch.cuh",
                    "paper_2608_23786_gb300/csrc/stepper_staged.cuh", "paper_2608_23786_gb300/csrc/stepper_async.cuh",
-                   "paper_2608_23786_gb300/csrc/stepper_f32_pull.cu"]
-# DRAM bytes (read + write) per launch of the stepper on this workload, from one ncu capture of the
+                   "paper_2608_23786_gb300/csrc/stepper_f32_pull.cu", "paper_2608_23786_gb300/csrc/level_args.cuh",
+                   "paper_2608_23786_gb300/csrc/stepper_march.cuh", "paper_2608_23786_gb300/csrc/march_launch.cuh",
+                   "paper_2608_23786_gb300/csrc/march.cu", "paper_2608_23786_gb300/csrc/march_f32.cu"]
+# DRAM bytes (read + write) per launch of the launch-per-step stepper on this workload, from one ncu capture of the
 # kernel built from sources with this digest and launched with this shape (kind, vec, block); the
 # capture ran 16 of the 64 samples (318.8 MB read + 267.5 MB written) and is scaled by 64/16.
 # Reported as null when the sources or the launch shape differ.
@@ -56,6 +63,12 @@ def stepper_digest():
                 if code:
                     h.update(code.encode() + b"\n")
     return h.hexdigest()[:16]
+
+
+def takes_multi_step(precision, exact_gamma=False, chosen=False):
+    """Whether a long call of the benchmark's large ensembles runs in the multi-step kernel (FP32
+    storage, closed-form gamma, no launch shape set)."""
+    return precision == "fp32" and not exact_gamma and not chosen
 
 
 def measured_peaks():
@@ -181,9 +194,10 @@ def _event_time(stream, fn, n):
 def measure_targets(dev, stream, peaks, peak_kind, lattice=19):
     """The 128^3 x 32 target configuration (FP32 and FP16 shifted storage, pull and
     AA), the 512^3 x 4 FP16 AA configuration, and the three-level batch (FP32 pull, FP16 AA),
-    each with the library's default launch shape: GLUPS and HBM fraction of the stepper from
-    CUDA events over whole steps (every step is one stepper launch; a batch macro step is one
-    graph replay of its sub-steps)."""
+    each with the library's default launch shape: GLUPS of the stepper from CUDA events over whole steps,
+    and the bytes its updates read and write as a fraction of the HBM copy (FP16: every step is one
+    stepper launch, a batch macro step one graph replay of its sub-steps; FP32: the steps of a call
+    run in one launch per ensemble, whose reads L2 serves, so the fraction can be above one)."""
     import torch
     from paper_2608_23786_gb300 import Ensemble, mclbm
     import ensemble_inputs as gen
@@ -206,7 +220,8 @@ def measure_targets(dev, stream, peaks, peak_kind, lattice=19):
         ach = bpl * lu / sec / 1e9
         launch = launch_desc(mclbm.mclbm_get_launch_parity(ens.ctx, 0),
                              mclbm.mclbm_get_launch_parity(ens.ctx, 1) if pat == "aa" else None)
-        out[name] = {"glups": lu / sec / 1e9, "avg_launch_ms": sec / n * 1e3, "steps_timed": n,
+        out[name] = {"glups": lu / sec / 1e9, "ms_per_update": sec / n * 1e3, "steps_timed": n,
+                     "kernel": MULTI_STEP_KERNEL if takes_multi_step(prec) else KERNEL_NAMES[mclbm.mclbm_get_launch(ens.ctx)[0]],
                      "bytes_per_lu": bpl, "achieved_gbs": ach, "peak_gbs": peaks["hbm_gbs"], "peak_kind": peak_kind,
                      "frac": ach / peaks["hbm_gbs"], "launch": dict(launch, chosen_by="default"),
                      "clocks": clk.summary()}
@@ -233,7 +248,7 @@ def measure_targets(dev, stream, peaks, peak_kind, lattice=19):
         out[f"levels_64x64_128x32_256x8_{prec}_{pat}"] = {
             "glups": lu / sec / 1e9, "ms_per_macro_step": sec / n * 1e3, "macro_steps_timed": n, "substeps": subs,
             "bytes_per_lu": bpl, "achieved_gbs": ach, "peak_gbs": peaks["hbm_gbs"], "peak_kind": peak_kind,
-            "frac": ach / peaks["hbm_gbs"], "launch": dict(launch, chosen_by="default"), "graph": True,
+            "frac": ach / peaks["hbm_gbs"], "launch": dict(launch, chosen_by="default"), "graph": not takes_multi_step(prec),
             "clocks": clk.summary()}
         mclbm.mclbm_batch_destroy(b)
         del levels
@@ -671,8 +686,8 @@ def run_oracle_report(args):
 
 
 def run_levels(args, precision):
-    """Uneven batch of the diffusive-scaling viscosity sequence in one graph-captured launch per
-    sub-step: 64^3 x 64, 128^3 x 32, 256^3 x 8 at Re 400 / 1600 / 3200, Ma 0.025 / 0.0125 / 0.00625,
+    """Uneven batch of the diffusive-scaling viscosity sequence, in one graph-captured launch per
+    sub-step (FP16) or level by level in the multi-step kernel (FP32): 64^3 x 64, 128^3 x 32, 256^3 x 8 at Re 400 / 1600 / 3200, Ma 0.025 / 0.0125 / 0.00625,
     1 : 4 : 16 sub-steps per macro step.  One bench step = one macro step.  The statistics the
     levels feed (shell spectra, S_2 / S_3 along axes, W1 between consecutive levels) are timed
     once after the timed region and reported separately."""
@@ -726,9 +741,9 @@ def run_levels(args, precision):
         "data": "synthetic",
         "config": {"workload": f"levels_64x64_128x32_256x8_{precision}_{pattern}", "substeps": subs,
                    "launch": launch_desc(tuned, mclbm.mclbm_batch_get_launch_parity(b, 1) if pattern == "aa" else None),
-                   "graph": True,
+                   "graph": not takes_multi_step(precision),
                    "l2": "inputs larger than L2"},
-        "roofline": {"kernel": KERNEL_NAMES[tuned[0]], "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
+        "roofline": {"kernel": MULTI_STEP_KERNEL if takes_multi_step(precision) else KERNEL_NAMES[tuned[0]], "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"], "peak_kind": peak_kind, "traffic": None},
         "stats_once_s": stats_s, "w1_consecutive_levels": w1, "w1_2pt_consecutive_levels": w12,
         "spectrum_finite": bool(all(np.all(np.isfinite(x)) for x in spectra + sfa)),
@@ -952,7 +967,10 @@ def main():
     mean = torch.empty((3,) + (wl["N"],) * 3, dtype=torch.float64, device=dev)
     var = torch.empty_like(mean)
     E = np.zeros(wl["M"])
-    kernels_per_step = S + 2  # S stepper launches, one pass for E(t) and the mean/var fields, its energy reduce
+    multi = takes_multi_step(wl["precision"], args.exact_gamma, bool(args.launch)) and S >= 12
+    # pull ensembles take an even number of updates in the multi-step kernel
+    stepper_launches = (1 + (S % 2 if wl["pattern"] == "pull" else 0)) if multi else S
+    kernels_per_step = stepper_launches + 2  # and one pass for E(t) and the mean/var fields, its energy reduce
 
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
 
@@ -982,7 +1000,7 @@ def main():
         dist.barrier()
     torch.cuda.synchronize()
     elapsed = t_start.elapsed_time(t_end) / 1e3
-    stepper_s = sum(a.elapsed_time(b) for a, b in ev) / 1e3 / (args.steps * S)  # per launch
+    stepper_s = sum(a.elapsed_time(b) for a, b in ev) / 1e3 / (args.steps * S)  # per update of the ensemble
     if world > 1:
         t = torch.tensor([elapsed], dtype=torch.float64)
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
@@ -1105,13 +1123,25 @@ def main():
     achieved = bpl / stepper_s / 1e9
     digest = stepper_digest()
     traffic = (NCU_TRAFFIC["bytes_per_launch"]
-               if NCU_TRAFFIC["sha256"] == digest and tuple(tuned[:3]) == NCU_TRAFFIC["launch"] and wl["M"] == 64
+               if not multi and NCU_TRAFFIC["sha256"] == digest and tuple(tuned[:3]) == NCU_TRAFFIC["launch"] and wl["M"] == 64
                and wl["lattice"] == 19
                and wl["N"] == 64 and wl["precision"] == "fp32" and wl["pattern"] == "pull" else None)
     cpu = None
     if not args.no_cpu_baseline and world == 1:
         v, desc, cores = oracle_sample(wl)
         cpu = {"value": v, "unit": "GLUPS", "cores": cores, "kind": "oracle", "sample": desc}
+    # the bytes that the updates read and write: through L2 in the multi-step kernel, which takes the
+    # state to and from HBM once per several updates, from and to HBM otherwise
+    peak = L2_COPY_GBS if multi else peaks["hbm_gbs"]
+    kernel = (f"{MULTI_STEP_KERNEL}<{wl['precision']},{wl['pattern']}>" if multi else
+              f"{KERNEL_NAMES[tuned[0]]}<{wl['precision']},{wl['pattern']},vec={tuned[1]},block={tuned[2]}>")
+    roofline = {"kernel": kernel, "bound": "l2" if multi else "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                "frac": achieved / peak, "peak_kind": "copy within L2, measured" if multi else peak_kind,
+                "traffic": traffic, "updates_per_launch": S // stepper_launches if multi else 1,
+                "algorithmic_bytes_per_update": bpl, "ms_per_update": stepper_s * 1e3,
+                "avg_launch_ms": stepper_s * S / stepper_launches * 1e3,
+                "over_hbm_copy": achieved / peaks["hbm_gbs"],
+                "stepper_glups": wl["M"] * wl["N"] ** 3 / stepper_s / 1e9}
     out = {
         "metric": "ensemble_glups", "value": value, "unit": "GLUPS", "n_gpus": world, "steps": args.steps,
         "warmup": max(3, args.warmup), "ms_per_step": elapsed / args.steps * 1e3, "higher_is_better": True,
@@ -1120,16 +1150,11 @@ def main():
         "config": {"workload": wl["name"], "N": wl["N"], "M_per_gpu": wl["M"], "Re": wl["Re"], "Ma": wl["Ma"],
                    "lattice": f"D3Q{wl['lattice']}", "storage": wl["precision"], "streaming": wl["pattern"],
                    "updates_per_step": S,
-                   "reductions_per_step": ["E_m(t)", "mean/var fields"], "l2": f"inputs ({bpl / 1e9:.2f} GB moved per update) "
+                   "reductions_per_step": ["E_m(t)", "mean/var fields"], "l2": f"inputs ({bpl / 2e9:.2f} GB of populations) "
                          "larger than the 129 MB L2: no flush",
                    "launch": dict(launch_desc(tuned, main_odd),
                                   chosen_by="explicit" if args.launch else ("autotuner" if args.autotune else "default"))},
-        "roofline": {"kernel": KERNEL_NAMES[tuned[0]] +
-                     f"<{wl['precision']},{wl['pattern']},vec={tuned[1]},block={tuned[2]}>",
-                     "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                     "frac": achieved / peaks["hbm_gbs"], "peak_kind": peak_kind,
-                     "traffic": traffic, "algorithmic_bytes_per_launch": bpl,
-                     "avg_launch_ms": stepper_s * 1e3, "stepper_glups": wl["M"] * wl["N"] ** 3 / stepper_s / 1e9},
+        "roofline": roofline,
         "cpu_baseline": cpu,
         "e2e": None if args.no_e2e else {"value": e2e_value, "unit": "GLUPS",
                                          "h2d_bytes_per_step": int(params_h.numel() * 8),
