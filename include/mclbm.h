@@ -168,8 +168,8 @@ MCLBM_API int mclbm_get_params(const mclbm_ctx* ctx, double* params);
 
 /* Advance every sample by nsteps fused stream+collide steps (Eq. (lbIteration)
  * with the KBC collision Eq. (kbcCollision) and the closed-form stabiliser
- * Eq. (entropyControl)).  Calls of several steps on FP32 storage, and on FP16 storage of small
- * ensembles, run as one launch that keeps the lattice planes in work in L2 (the same results;
+ * Eq. (entropyControl)).  Calls of several steps on FP32 storage, and on FP16 and FP64 storage of
+ * small ensembles, run as one launch that keeps the lattice planes in work in L2 (the same results;
  * unless mclbm_set_launch has chosen a shape).
  * Enqueued only.  Errors: INVALID_ARG, CUDA. */
 MCLBM_API int mclbm_step(mclbm_ctx* ctx, int64_t nsteps);

@@ -9,6 +9,7 @@ namespace mclbm {
 
 cudaError_t launch_march_f32(MarchArgs<float>& a, int vec, int mode, int num_sms, int64_t tiles, cudaStream_t s);
 cudaError_t launch_march_f16(MarchArgs<__half>& a, int vec, int mode, int num_sms, int64_t tiles, cudaStream_t s);
+cudaError_t launch_march_f64(MarchArgs<double>& a, int vec, int mode, int num_sms, int64_t tiles, cudaStream_t s);
 
 namespace {
 
@@ -92,11 +93,18 @@ bool march_order(MarchArgs<E>& a, const mclbm_ctx* c, int vec, int64_t steps)
 // FP16 storage is bound by arithmetic, in a kernel with twice the nodes per thread (65 against 78 GLUPS
 // at 64^3 x 64): here only what is bound by launches and latency, 6.2 against 2.4 to 3.5 us per step up
 // to 32^3, 64^3 8.3 against 5.2, 64^3 x 4 18.5 against 16.4 (D3Q27 64^3 x 2 14.4 against 13.2 us).
-// FP64 storage is bound by its arithmetic from 32^3 on.
+//
+// FP64 storage is bound by its pipe: a warp's collision holds a partition for 12 us, so a launch per
+// step takes whole multiples of that (32^3: 1024 warps on 608 partitions) and the launch's 2 to 3 us.
+// Without a barrier between the steps the partitions fill evenly: 32^3 26.7 -> 25.2 us per step, x 2
+// 49.2 -> 39.2, x 3 71.8 -> 58.4, x 4 84.0 -> 77.8, x 8 164 -> 156, x 16 316 -> 312 (x 32 no gain: 627 and
+// 625), 16^3 15.9 -> 14.2, 8^3 14.4 -> 13.9; D3Q27 32^3 x 2 69.6 -> 55.7.  Eight steps: 32^3 27.2 against
+// 27.2, x 2 49.9 against 41.5, 8^3 15.0 against 15.2.  Rows within one warp only (N <= 32).
 bool march_serves(const mclbm_ctx* c, int64_t steps)
 {
-    if (c->cfg.precision == MCLBM_FP64 || (c->cfg.options & MCLBM_OPT_EXACT_GAMMA) || c->launch_chosen) return false;
+    if ((c->cfg.options & MCLBM_OPT_EXACT_GAMMA) || c->launch_chosen) return false;
     const int64_t nodes = (int64_t)c->M * c->n;
+    if (c->cfg.precision == MCLBM_FP64) return c->N <= 32 && nodes <= 1 << 19 && steps >= (nodes <= (1 << 15) ? 16 : 8);
     if (c->cfg.precision == MCLBM_FP16) return steps >= 6 && nodes <= (Q == 19 ? 1 << 20 : 1 << 19);
     return steps >= (nodes < (1 << 16) ? 12 : (nodes < (1 << 18) ? 6 : 3));
 }
@@ -108,6 +116,7 @@ bool march_serves(const mclbm_ctx* c, int64_t steps)
 // four and the four ahead spill, always (64^3 x 2 13.5 -> 13.2).  D3Q27 FP32 rows that span warps: two.
 int march_vec(int precision, int N, int64_t nodes)
 {
+    if (precision == MCLBM_FP64) return 1;  // as the launch per step of small ensembles
     if (Q == 27) return precision == MCLBM_FP16 || nodes <= (1 << 18) || N > 128 ? 2 : 4;
     return nodes <= (precision == MCLBM_FP32 ? 1 << 18 : 1 << 17) ? 2 : 4;
 }
@@ -143,7 +152,9 @@ cudaError_t march_t(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t 
         }
         cudaError_t e = cudaMemsetAsync(a.cnt, 0, cnt_bytes, c->stream);
         if (e != cudaSuccess) return e;
-        if constexpr (f32)
+        if constexpr (std::is_same<E, double>::value)
+            e = launch_march_f64(a, vec, mode, c->num_sms, tiles, c->stream);
+        else if constexpr (f32)
             e = launch_march_f32(a, vec, mode, c->num_sms, tiles, c->stream);
         else
             e = launch_march_f16(a, vec, mode, c->num_sms, tiles, c->stream);
@@ -155,6 +166,15 @@ cudaError_t march_t(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t 
         *taken += k;
     }
     return cudaSuccess;
+}
+
+cudaError_t march_any(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t hop, int64_t nsteps, int64_t* taken)
+{
+    switch (c->cfg.precision) {
+        case MCLBM_FP64: return march_t<double>(c, mode, src, dst, hop, nsteps, taken);
+        case MCLBM_FP32: return march_t<float>(c, mode, src, dst, hop, nsteps, taken);
+        default: return march_t<__half>(c, mode, src, dst, hop, nsteps, taken);
+    }
 }
 
 }  // namespace
@@ -171,8 +191,7 @@ cudaError_t launch_march(mclbm_ctx* c, int64_t nsteps, int64_t* taken)
     *taken = 0;
     const int mode = c->cfg.pattern == MCLBM_PULL ? kMarchSwap : kMarchAA;
     if (!march_serves_call(c, nsteps)) return cudaSuccess;
-    const cudaError_t e = c->cfg.precision == MCLBM_FP32 ? march_t<float>(c, mode, nullptr, nullptr, 0, nsteps, taken)
-                                                         : march_t<__half>(c, mode, nullptr, nullptr, 0, nsteps, taken);
+    const cudaError_t e = march_any(c, mode, nullptr, nullptr, 0, nsteps, taken);
     c->steps += *taken;
     return e;
 }
@@ -185,8 +204,7 @@ cudaError_t launch_march_trajectory(mclbm_ctx* c, const void* src, void* dst, si
     *taken = 0;
     if (!march_serves(c, nsteps)) return cudaSuccess;
     const int64_t hop = (int64_t)(hop_bytes / c->elem_bytes);
-    return c->cfg.precision == MCLBM_FP32 ? march_t<float>(c, kMarchTrajectory, src, dst, hop, nsteps, taken)
-                                          : march_t<__half>(c, kMarchTrajectory, src, dst, hop, nsteps, taken);
+    return march_any(c, kMarchTrajectory, src, dst, hop, nsteps, taken);
 }
 
 }  // namespace mclbm

@@ -1,4 +1,4 @@
-"""Calls of several steps on FP32 and (small) FP16 storage (one launch of the multi-step kernel) against the same steps
+"""Calls of several steps on FP32 and (small) FP16 and FP64 storage (one launch of the multi-step kernel) against the same steps
 taken one call at a time (a launch per step): the same bits, for both streaming patterns, one and
 several tiles per plane, several planes per tile, windows and whole lattices in L2, even and odd
 step counts and a state at an odd step."""
@@ -43,6 +43,17 @@ def test_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
 @pytest.mark.parametrize("N,M,steps", [(8, 1, 7), (16, 3, 6), (32, 4, 8), (32, 7, 9), (64, 2, 6)])
 def test_fp16_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
     a, b = _pair(N, M, "fp16", pattern=pattern, lattice=lattice)
+    a.step(steps)
+    for _ in range(steps):
+        b.step(1)
+    _same(a, b)
+
+
+@pytest.mark.parametrize("lattice", [19, 27])
+@pytest.mark.parametrize("pattern", ["pull", "aa"])
+@pytest.mark.parametrize("N,M,steps", [(8, 1, 16), (8, 131, 9), (16, 3, 17), (32, 1, 17), (32, 5, 8), (32, 16, 8)])
+def test_fp64_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
+    a, b = _pair(N, M, "fp64", pattern=pattern, lattice=lattice)
     a.step(steps)
     for _ in range(steps):
         b.step(1)
