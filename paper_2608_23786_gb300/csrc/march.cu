@@ -91,8 +91,12 @@ bool march_order(MarchArgs<E>& a, const mclbm_ctx* c, int vec, int64_t steps)
 // us, 32^3 x 3 23.3 against 25.1 us.
 //
 // FP16 storage is bound by arithmetic, in a kernel with twice the nodes per thread (65 against 78 GLUPS
-// at 64^3 x 64): here only what is bound by launches and latency, 6.2 against 2.4 to 3.5 us per step up
-// to 32^3, 64^3 8.3 against 5.2, 64^3 x 4 18.5 against 16.4 (D3Q27 64^3 x 2 14.4 against 13.2 us).
+// at 64^3 x 64): here only what is bound by launches, latency and unfilled waves.  6.2 against 2.4 to 3.5 us
+// per step up to 32^3, 64^3 8.3 against 5.2, 64^3 x 4 18.5 against 16.0, x 5 22.4 against 20.0, x 8 33.0
+// against 31.9, AA 33.9 against 31.3; beyond, waves fill (x 10 39.6 against 40).  D3Q27, whose two nodes
+// per thread reach 40 GLUPS: 64^3 x 2 14.4 against 13.2, AA 16.4 against 12.9, 64^3 x 3 20.6 against 19.7,
+// AA 22.0 against 19.3, 32^3 x 25 20.6 in both, AA 22.6 against 19.9, 64^3 x 4 AA 25.7 in both.  Twelve
+// steps: 64^3 x 8 33.4 against 32.8, D3Q27 64^3 x 3 20.84 against 20.82; six steps of those lose 1 to 5%.
 //
 // FP64 storage is bound by its pipe: a warp's collision holds a partition for 12 us, so a launch per
 // step takes whole multiples of that (32^3: 1024 warps on 608 partitions) and the launch's 2 to 3 us.
@@ -105,7 +109,11 @@ bool march_serves(const mclbm_ctx* c, int64_t steps)
     if ((c->cfg.options & MCLBM_OPT_EXACT_GAMMA) || c->launch_chosen) return false;
     const int64_t nodes = (int64_t)c->M * c->n;
     if (c->cfg.precision == MCLBM_FP64) return c->N <= 32 && nodes <= 1 << 19 && steps >= (nodes <= (1 << 15) ? 16 : 8);
-    if (c->cfg.precision == MCLBM_FP16) return steps >= 6 && nodes <= (Q == 19 ? 1 << 20 : 1 << 19);
+    if (c->cfg.precision == MCLBM_FP16) {
+        if constexpr (Q == 19) return nodes <= 1 << 20 ? steps >= 6 : steps >= 12 && nodes <= 1 << 21;
+        if (nodes <= 1 << 18) return steps >= 6;
+        return steps >= 12 && nodes <= (c->cfg.pattern == MCLBM_PULL ? 6 : 7) << 17;
+    }
     return steps >= (nodes < (1 << 16) ? 12 : (nodes < (1 << 18) ? 6 : 3));
 }
 

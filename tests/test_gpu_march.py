@@ -40,7 +40,8 @@ def test_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
 
 @pytest.mark.parametrize("lattice", [19, 27])
 @pytest.mark.parametrize("pattern", ["pull", "aa"])
-@pytest.mark.parametrize("N,M,steps", [(8, 1, 7), (16, 3, 6), (32, 4, 8), (32, 7, 9), (64, 2, 6)])
+@pytest.mark.parametrize("N,M,steps", [(8, 1, 7), (16, 3, 6), (32, 4, 8), (32, 7, 9), (64, 2, 6), (64, 3, 13),
+                                       (128, 1, 12)])
 def test_fp16_several_steps_equal_single_steps(N, M, steps, pattern, lattice):
     a, b = _pair(N, M, "fp16", pattern=pattern, lattice=lattice)
     a.step(steps)
