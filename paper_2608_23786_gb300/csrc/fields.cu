@@ -167,9 +167,11 @@ __global__ void k_reduce_rows(const double* __restrict__ partial, int rows, int 
 // x 32 FP16 pull 3011 -> 674 us) or which are bound elsewhere.  FP64 operations per node beyond the
 // samples' (GB300's FP64 units bound few samples on a large lattice: 256^3 x 8 FP16 AA): 15, the
 // conversions by integer operations.  256^3 x 8 FP16 AA 1674 -> 1475 us (odd steps 2124 -> 1556), 16^3 x 100
-// FP16 348 -> 156, 64^3 x 8 FP64 415 -> 369.
+// FP16 348 -> 156, 64^3 x 8 FP64 415 -> 369.  D3Q27 FP16, whose run of four and the one in flight do not
+// fit the registers, takes two nodes: 16^3 x 200 192 us with element loads, 243 with four nodes, 136 with
+// two; 64^3 x 64 369 -> 242 (two).
 template <class E>
-constexpr int kRunVec = sizeof(E) == 2 ? 4 : 2;
+constexpr int kRunVec = sizeof(E) == 2 && Q == 19 ? 4 : 2;
 template <class E>
 constexpr bool kRunScalar = sizeof(E) == 4;
 constexpr int kSampleChunk = 8;
