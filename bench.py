@@ -1152,7 +1152,8 @@ def main():
                    "updates_per_step": S,
                    "reductions_per_step": ["E_m(t)", "mean/var fields"], "l2": f"inputs ({bpl / 2e9:.2f} GB of populations) "
                          "larger than the 129 MB L2: no flush",
-                   "launch": dict(launch_desc(tuned, main_odd),
+                   # the shape where an update is a launch
+                   "launch": dict({"kind": "multi_step"} if multi else launch_desc(tuned, main_odd),
                                   chosen_by="explicit" if args.launch else ("autotuner" if args.autotune else "default"))},
         "roofline": roofline,
         "cpu_baseline": cpu,
