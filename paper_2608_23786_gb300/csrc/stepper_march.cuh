@@ -246,6 +246,9 @@ __device__ __forceinline__ void march_hand_out(const MarchArgs<E>& a, MarchShare
             __nanosleep(kMarchNapNs);
             if ((it & 63) == 0 && __any_sync(0xffffffffu, lane == 0 && march_give_up(t0, a.err))) return;
         }
+        // Lanes 0, 1 and 2 each acquired one counter; a vote orders no memory, so without this lane 0's
+        // release would not carry what lanes 1 and 2 acquired.
+        __syncwarp();
         if (lane == 0) {
             sh.tile[g][n & (2 * kMarchAhead - 1)] = t;
             if (!t.valid) st_release_cta(smem_u32(&sh.last[g]), n);
