@@ -170,6 +170,9 @@ __global__ void k_reduce_rows(const double* __restrict__ partial, int rows, int 
 // FP16 348 -> 156, 64^3 x 8 FP64 415 -> 369.  D3Q27 FP16, whose run of four and the one in flight do not
 // fit the registers, takes two nodes: 16^3 x 200 192 us with element loads, 243 with four nodes, 136 with
 // two; 64^3 x 64 369 -> 242 (two).
+// Stores: 16 bytes where both fields are aligned, but FP32 element by element: with the second form of
+// store in its kernel the loop over the samples runs slower (energies wanted, with / without: 64^3 x 64 304 /
+// 274 us, 64^3 x 16 118 / 107, 32^3 x 200 381 / 329; without energies 64^3 x 4 35.0 / 33.2, 256^3 x 2 962 / 974).
 template <class E>
 constexpr int kRunVec = sizeof(E) == 2 && Q == 19 ? 4 : 2;
 template <class E>
@@ -329,10 +332,10 @@ __global__ void __launch_bounds__(kStatsThreads<E>) k_stats_pass(const E* __rest
                     vv[h] = fma(-s1[a][k + h] * invM, s1[a][k + h], s2[a][k + h]) * vscale;
                 }
                 double *mo = mean + a * g.n + node + k, *vo = var + a * g.n + node + k;
-                if (pairs) {
+                if (!kRunScalar<E> && pairs) {
                     vstore<double, 2>(mo, mv);
                     vstore<double, 2>(vo, vv);
-                } else {  // the caller's fields are not 16-byte aligned
+                } else {  // FP32, or the caller's fields are not 16-byte aligned
                     mo[0] = mv[0], mo[1] = mv[1];
                     vo[0] = vv[0], vo[1] = vv[1];
                 }
