@@ -259,7 +259,8 @@ MCLBM_API int mclbm_w1_restricted(const double* d_a, int32_t MA, const double* d
  * metric, every point pair i <= j, off-diagonal pairs counted twice, divided by G^2.  Each
  * pair is an exact transport problem between uniform empirical measures (1 <= MA, MB <= 1024):
  * for L = lcm(MA, MB) <= 256 an assignment of L atoms per side (atoms repeated L/MA, L/MB
- * times), one warp per problem; otherwise the transportation problem with integer supply MB/g
+ * times), one warp per problem; for larger L, and for unequal counts whose repetition costs more than
+ * it saves (L > 64 and few problems or many copies), the transportation problem with integer supply MB/g
  * per atom of A and demand MA/g per atom of B (g = gcd(MA, MB)) by successive shortest paths,
  * one block per problem.  Costs are fixed-point integers from FP32 atoms taken relative to
  * their mean; the plan is optimal for those costs and its cost is summed in FP64 (each pair's

@@ -16,7 +16,8 @@
 //    times gives uniform weights 1/L on both sides without changing the optimum, and an optimal
 //    plan is then a permutation: one warp solves the L x L assignment problem with the
 //    shortest-augmenting-path (Hungarian) method after a column reduction, each lane owning up to
-//    eight columns.
+//    eight columns.  Unequal counts whose repetition makes the problem much larger are left to the
+//    second solver (match_serves).
 //  - otherwise (M_A, M_B <= 1024): one block solves the transportation problem directly, with
 //    g = gcd(M_A, M_B), integer supply M_B / g at every atom of A and demand M_A / g at every atom
 //    of B (the plan pi = x / (M_A M_B / g)), by successive shortest paths: rows (atoms of A) are
@@ -361,7 +362,7 @@ __global__ void __launch_bounds__(32 * kPairWarps) k_w1_match(const double* __re
     }
 }
 
-// ---- transportation problems beyond the warp kernel (L > 256): one block per problem -----------------
+// ---- transportation problems beyond the warp kernel (match_serves): one block per problem -----------------
 constexpr int kTpMaxM = 1024;          // atoms per side
 constexpr int kTpThreads = 256;        // threads per block
 constexpr int kTpWarps = kTpThreads / 32;
@@ -751,6 +752,22 @@ int gcd_int(int a, int b)
     return a;
 }
 
+// Whether the warp kernel takes the problems (else the block solver).  Unequal counts: the L x L problem
+// has c = (L / MA)(L / MB) times the entries of the MA x MB one, and equal atoms lengthen its searches, which
+// the block solver does not repeat; the warp kernel, for its part, solves seven times as many problems at
+// once and takes longer for one.  Measured warp / block time against c L (1, 36, 378, 2080 and 23,436
+// vector problems): 100, 50 (200) 0.41, 0.48, 0.3, 0.1, -; 24, 36 (432) 0.53, 0.74, 0.42, 0.13, 0.09; 256, 128
+// (512) 1.02, 1.07, 0.5, 0.25, -; 250, 50 (1250) 1.7, 1.7, 0.95, 0.46, 0.27; 100, 40 (2000) 2.4, 2.6, 1.3, 0.6,
+// 0.4; 256, 16 (4096) 2.8, 2.8, 1.4, 0.7, 0.5; 10, 7 (4900) 3.2, 3.4, 2.5, 0.98, 0.73; 12, 11 (17,424) 8.4, 9.5,
+// 5.5, 3.0, 2.0; 16, 15 (57,600) 20, 22, 13, 6.3, -.  Equal counts: below 0.8 throughout.
+bool match_serves(int MA, int MB, int64_t L, int64_t nprob)
+{
+    if (L > kPairMaxL) return false;
+    if (L <= 64 || MA == MB) return true;
+    const int64_t size = L / MA * (L / MB) * L;
+    return size <= 5000 && size <= 400 + 2 * nprob;
+}
+
 }  // namespace
 
 // Work buffer: per-problem values [nprob], partial sums [kPairParts], the total and an error
@@ -770,7 +787,7 @@ PairWork pair_work(int MA, int MB, int G, int vector)
     w.flows = (w.err + 16 + 255) / 256 * 256;
     const int g = gcd_int(MA, MB);
     const int64_t L = (int64_t)MA / g * MB;
-    const bool general = L > 64 && MA != MB;
+    const bool general = L > 64 && MA != MB;  // whichever solver the number of problems chooses
     const size_t fstride = ((size_t)MA * MB + 7) / 8 * 8;  // elements per block, as in the kernel
     w.bytes = w.flows + (general ? (size_t)kTpGeneralBlocks * fstride * sizeof(unsigned short) : 0);
     return w;
@@ -813,7 +830,7 @@ int mclbm_w1_2pt(const double* d_a, int32_t MA, const double* d_b, int32_t MB, i
     MCLBM_CUDA(cudaGetDevice(&dev));
     MCLBM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     MCLBM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    if (L <= kPairMaxL) {
+    if (match_serves(MA, MB, L, nprob)) {
         auto launch = [&](auto kernel, int K) -> cudaError_t {
             const int smem = kPairWarps * match_smem(K, (int)L);
             cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
