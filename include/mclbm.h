@@ -270,7 +270,9 @@ MCLBM_API int mclbm_w1_restricted(const double* d_a, int32_t MA, const double* d
  * mclbm_w1_2pt_work_bytes(MA, MB, G, vector) bytes, 256-byte aligned (it includes, for unequal
  * MA and MB with lcm > 64, one 2 MA MB-byte flow matrix for each of 256 problems in flight).
  * Runs on cuda_stream and synchronises it.  Errors: INVALID_ARG, SHAPE (MA or MB > 1024),
- * OOM (work buffer too small), NONFINITE (a search failed, e.g. on non-finite atoms). */
+ * OOM (work buffer too small), NONFINITE (a problem has no finite value: non-finite atoms,
+ * or atoms so far apart, above 1e18, that no plan has finite FP32 costs; W and d_per_pair then hold NaN or
+ * Inf for the problems concerned). */
 MCLBM_API size_t mclbm_w1_2pt_work_bytes(int32_t MA, int32_t MB, int32_t G, int32_t vector);
 MCLBM_API int mclbm_w1_2pt(const double* d_a, int32_t MA, const double* d_b, int32_t MB, int32_t G, int32_t vector,
                            void* d_work, size_t work_bytes, void* cuda_stream, double* W, double* d_per_pair);

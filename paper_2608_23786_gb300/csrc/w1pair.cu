@@ -27,8 +27,10 @@
 //    counts are assignment problems again (supply and demand 1): the matching is kept in shared
 //    memory.  Otherwise the integer flows x_ij (at most min(supply, demand) <= 1024, 16 bits) are
 //    kept in a column-major matrix in the work buffer, one per block in flight.
+#include <math_constants.h>
+
+#include <cfloat>
 #include <cmath>
-#include <cstring>
 #include <string>
 
 #include "internal.h"
@@ -95,7 +97,7 @@ __device__ __forceinline__ double cost64(const double* A, const double* B, int G
 }
 
 template <int K>
-__device__ __forceinline__ long long qcost(const float (&x)[K], const float (&y)[K], float scale)
+__device__ __forceinline__ float dist2(const float (&x)[K], const float (&y)[K])
 {
     float s = 0.f;
 #pragma unroll
@@ -103,7 +105,13 @@ __device__ __forceinline__ long long qcost(const float (&x)[K], const float (&y)
         const float e = x[d] - y[d];
         s = fmaf(e, e, s);
     }
-    return __float2ll_rn(sqrtf(s) * scale);
+    return s;
+}
+
+template <int K>
+__device__ __forceinline__ long long qcost(const float (&x)[K], const float (&y)[K], float scale)
+{
+    return __float2ll_rn(sqrtf(dist2<K>(x, y)) * scale);
 }
 
 // The fixed-point cost as qcost forms it, without the 64-bit conversion (16 results per SM and clock
@@ -112,13 +120,7 @@ __device__ __forceinline__ long long qcost(const float (&x)[K], const float (&y)
 template <int K>
 __device__ __forceinline__ long long qcost_split(const float (&x)[K], const float (&y)[K], float scale)
 {
-    float s = 0.f;
-#pragma unroll
-    for (int d = 0; d < K; ++d) {
-        const float e = x[d] - y[d];
-        s = fmaf(e, e, s);
-    }
-    const float c = sqrtf(s) * scale;
+    const float c = sqrtf(dist2<K>(x, y)) * scale;
     constexpr float kMagic = 12582912.0f;  // 1.5 2^23
     constexpr int kMagicBits = 0x4B400000;
     const float h = __fmaf_rn(c, 9.5367431640625e-7f, kMagic);
@@ -157,8 +159,7 @@ __host__ __device__ inline int match_smem(int K, int L)  // bytes per warp
 template <int K, int CPL>
 __global__ void __launch_bounds__(32 * kPairWarps) k_w1_match(const double* __restrict__ A, int MA,
                                                               const double* __restrict__ B, int MB, int G, int L,
-                                                              int ncomp, int64_t nprob, double* __restrict__ per,
-                                                              int* __restrict__ err)
+                                                              int ncomp, int64_t nprob, double* __restrict__ per)
 {
     extern __shared__ __align__(16) unsigned char msm[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(32 * kPairWarps) k_w1_match(const double* __re
                 const unsigned mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
                 const int wl = __ffs(__ballot_sync(0xffffffffu, hi == mhi && lo == mlo)) - 1;
                 dcur = (long long)(((unsigned long long)mhi << 32) | mlo);
-                if (dcur >= kInf) break;  // nothing reachable: reported below
+                if (dcur >= kInf) break;  // nothing reachable: NaN below
                 const int j = 32 * __shfl_sync(0xffffffffu, bc, wl) + wl;
                 i = pcol[j];
                 if (i < 0) {
@@ -345,19 +346,23 @@ __global__ void __launch_bounds__(32 * kPairWarps) k_w1_match(const double* __re
             }
             __syncwarp();
         }
-        // W1 of the problem: mean FP64 cost of the matched pairs
+        // W1 of the problem: mean FP64 cost of the matched pairs; NaN if the search failed or if the plan
+        // holds a pair whose cost is no number in FP32 (qcost_split gives such costs a finite value
+        // above any other, so they are in a plan only where it cannot do without)
         double s = 0.0;
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
             const int col = lane + 32 * c;
-            if (col < L && pcol[col] >= 0) s += cost64<K>(A, B, G, pcol[col] / ra, col / rb, pb);
+            if (col < L) {
+                const int r = pcol[col];
+                if (r >= 0) s += cost64<K>(A, B, G, r / ra, col / rb, pb);
+                failed = failed || r < 0 || !(dist2<K>(row[r].x, y[c]) <= FLT_MAX);
+            }
         }
+        failed = __any_sync(0xffffffffu, failed);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) {
-            per[prob] = s / L;
-            if (failed) atomicExch(err, 1);
-        }
+        if (lane == 0) per[prob] = failed ? CUDART_NAN : s / L;
         __syncwarp();
     }
 }
@@ -446,15 +451,15 @@ __device__ __forceinline__ void tp_block_argmin(long long& best, int& bj, long l
 
 // One transportation problem per block (grid-strided over the problems).  MATCH: equal sample
 // counts (supply = demand = 1), matching in shared memory; otherwise the block's flow matrix
-// flowT [MB][MA] (column-major: the rows shipping to one column are contiguous).  err: set to 1
-// if a shortest-path search ends without reaching a column with open demand (it cannot while the
-// total supply equals the total demand; the check keeps every loop bounded).
+// flowT [MB][MA] (column-major: the rows shipping to one column are contiguous).  The problem's
+// value is NaN if a shortest-path search ends without reaching a column with open demand (with finite
+// costs it cannot while the total supply equals the total demand; the check keeps every loop bounded).
 template <int K, bool MATCH>
 __global__ void __launch_bounds__(kTpThreads, 2) k_w1_transport(const double* __restrict__ A, int MA,
                                                              const double* __restrict__ B, int MB, int G, int ncomp,
                                                              int64_t nprob, int supply, int demand,
                                                              unsigned short* __restrict__ flows,
-                                                             double* __restrict__ per, int* __restrict__ err)
+                                                             double* __restrict__ per)
 {
     extern __shared__ __align__(16) unsigned char tsm[];
     const TpLayout Lo = tp_layout(MA, MB, K);
@@ -700,10 +705,7 @@ __global__ void __launch_bounds__(kTpThreads, 2) k_w1_transport(const double* __
             }
         }
         s = tp_block_sum(s, sd);
-        if (tid == 0) {
-            per[prob] = s / (double)total_flow;
-            if (*s_fail) atomicExch(err, 1);
-        }
+        if (tid == 0) per[prob] = *s_fail ? CUDART_NAN : s / (double)total_flow;
         __syncthreads();
     }
 }
@@ -770,10 +772,9 @@ bool match_serves(int MA, int MB, int64_t L, int64_t nprob)
 
 }  // namespace
 
-// Work buffer: per-problem values [nprob], partial sums [kPairParts], the total and an error
-// word, then (unequal sample counts beyond the warp kernel) one flow matrix per block in flight.
+// Work buffer: per-problem values [nprob], partial sums [kPairParts] and the total, then (unequal sample counts beyond the warp kernel) one flow matrix per block in flight.
 struct PairWork {
-    size_t per, partial, total, err, flows, bytes;
+    size_t per, partial, total, flows, bytes;
 };
 
 PairWork pair_work(int MA, int MB, int G, int vector)
@@ -783,8 +784,7 @@ PairWork pair_work(int MA, int MB, int G, int vector)
     w.per = 0;
     w.partial = (size_t)nprob * sizeof(double);
     w.total = w.partial + kPairParts * sizeof(double);
-    w.err = w.total + 32 * sizeof(double);
-    w.flows = (w.err + 16 + 255) / 256 * 256;
+    w.flows = (w.total + 32 * sizeof(double) + 16 + 255) / 256 * 256;
     const int g = gcd_int(MA, MB);
     const int64_t L = (int64_t)MA / g * MB;
     const bool general = L > 64 && MA != MB;  // whichever solver the number of problems chooses
@@ -825,11 +825,9 @@ int mclbm_w1_2pt(const double* d_a, int32_t MA, const double* d_b, int32_t MB, i
     double* per = d_per_pair ? d_per_pair : (double*)(wb + pw.per);
     double* partial = (double*)(wb + pw.partial);
     double* total = (double*)(wb + pw.total);
-    int* err = (int*)(wb + pw.err);
     int dev = 0, sms = 0;
     MCLBM_CUDA(cudaGetDevice(&dev));
     MCLBM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    MCLBM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     if (match_serves(MA, MB, L, nprob)) {
         auto launch = [&](auto kernel, int K) -> cudaError_t {
             const int smem = kPairWarps * match_smem(K, (int)L);
@@ -841,7 +839,7 @@ int mclbm_w1_2pt(const double* d_a, int32_t MA, const double* d_b, int32_t MB, i
             if (per_sm < 1) return cudaErrorInvalidConfiguration;
             int64_t blocks = (nprob + kPairWarps - 1) / kPairWarps;
             if (blocks > (int64_t)sms * per_sm) blocks = (int64_t)sms * per_sm;
-            kernel<<<(unsigned)blocks, 32 * kPairWarps, smem, s>>>(d_a, MA, d_b, MB, G, (int)L, ncomp, nprob, per, err);
+            kernel<<<(unsigned)blocks, 32 * kPairWarps, smem, s>>>(d_a, MA, d_b, MB, G, (int)L, ncomp, nprob, per);
             return cudaGetLastError();
         };
         cudaError_t e;
@@ -873,7 +871,7 @@ int mclbm_w1_2pt(const double* d_a, int32_t MA, const double* d_b, int32_t MB, i
             if (!match && blocks > kTpGeneralBlocks) blocks = kTpGeneralBlocks;
             if (blocks > nprob) blocks = nprob;
             kernel<<<(unsigned)blocks, kTpThreads, smem, s>>>(d_a, MA, d_b, MB, G, ncomp, nprob, supply, demand, flows,
-                                                              per, err);
+                                                              per);
             return cudaGetLastError();
         };
         cudaError_t e;
@@ -887,15 +885,10 @@ int mclbm_w1_2pt(const double* d_a, int32_t MA, const double* d_b, int32_t MB, i
     k_pair_partials<<<kPairParts, kSumThreads, 0, s>>>(per, G, ncomp, nprob, chunk, partial);
     k_pair_total<<<1, 32, 0, s>>>(partial, kPairParts, 1.0 / ((double)G * G), total);
     MCLBM_CUDA(cudaGetLastError());
-    // the total and the error word lie 32 doubles apart: one copy brings both
-    double h_total[33];
-    MCLBM_CUDA(cudaMemcpyAsync(h_total, total, sizeof(h_total), cudaMemcpyDeviceToHost, s));
+    MCLBM_CUDA(cudaMemcpyAsync(W, total, sizeof(double), cudaMemcpyDeviceToHost, s));
     MCLBM_CUDA(cudaStreamSynchronize(s));
-    *W = h_total[0];
-    int h_err = 0;
-    memcpy(&h_err, &h_total[32], sizeof(int));
-    if (h_err)
-        return set_error(MCLBM_ERR_NONFINITE, "a transport search found no column with open demand (non-finite atoms?)");
+    if (!std::isfinite(*W))
+        return set_error(MCLBM_ERR_NONFINITE, "a transport problem has no finite value (non-finite atoms?)");
     return MCLBM_OK;
 }
 
