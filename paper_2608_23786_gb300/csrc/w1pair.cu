@@ -767,7 +767,7 @@ bool match_serves(int MA, int MB, int64_t L, int64_t nprob)
     if (L > kPairMaxL) return false;
     if (L <= 64 || MA == MB) return true;
     const int64_t size = L / MA * (L / MB) * L;
-    return size <= 5000 && size <= 400 + 2 * nprob;
+    return size <= 400 || (size <= 5000 && size <= 3 * nprob);
 }
 
 }  // namespace

@@ -31,7 +31,8 @@ def _gpu(ua, ub, vector):
     return W, per.cpu().numpy()
 
 
-# copies x L: 200; 432 (16 problems and fewer / more); 576; 1600 (600); 4900 (2250); 17424 and 57600 (never)
+# copies x L: 200 (always repeated); 432, 576 and 1600 (from 144, 192 and 534 problems on); 4900 (1634); 17424
+# and 57600 (never)
 @pytest.mark.parametrize("MA,MB", [(50, 100), (24, 36), (48, 32), (20, 16), (10, 7), (12, 11), (16, 15)])
 @pytest.mark.parametrize("G", [1, 5, 35])
 def test_both_routes_against_the_oracle(MA, MB, G):
