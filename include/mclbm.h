@@ -18,7 +18,9 @@
  *    256-byte aligned and stay valid until mclbm_destroy().
  *  - Every device call is enqueued on the CUDA stream given at creation (NULL =
  *    legacy default stream).  Calls that return host data synchronise that
- *    stream before returning; the others return as soon as work is enqueued.
+ *    stream before returning; the others return as soon as work is enqueued.  A call that
+ *    synchronises a context's stream returns MCLBM_ERR_TIMEOUT if a bounded device wait of the
+ *    stepper has given up since the context's last initialisation or load: its results then lack steps.
  *  - A context may be used by one host thread at a time; contexts on several
  *    devices may be used from one process.  A call on a context (or batch) runs on
  *    the context's device, the device current at mclbm_create: the call makes it
@@ -171,6 +173,9 @@ MCLBM_API int mclbm_get_params(const mclbm_ctx* ctx, double* params);
  * Eq. (entropyControl)).  Calls of several steps on FP32 storage, and on FP16 and FP64 storage of
  * small ensembles, run as one launch that keeps the lattice planes in work in L2 (the same results;
  * unless mclbm_set_launch has chosen a shape).
+ * That launch and the staged kernel wait within the device, each wait for a limited time; a wait that
+ * gives up leaves steps out of the state, which the next synchronising call on the context (and
+ * mclbm_device_status) reports as TIMEOUT until the next initialisation or load.
  * Enqueued only.  Errors: INVALID_ARG, CUDA. */
 MCLBM_API int mclbm_step(mclbm_ctx* ctx, int64_t nsteps);
 
@@ -384,7 +389,7 @@ MCLBM_API int mclbm_batch_autotune(mclbm_batch* b, int32_t trials, int32_t* kind
  * each segment is recomputed from its checkpoint.  Pull streaming only.  The context
  * must directly follow an initialisation; on return it holds the state at step nsteps.
  * d_buf: caller device buffer of mclbm_grad_required_bytes() bytes (256-aligned).
- * J [M], dJdX [M][24]: host.  Synchronises.  Errors: INVALID_ARG, OOM, CUDA. */
+ * J [M], dJdX [M][24]: host.  Synchronises.  Errors: INVALID_ARG, OOM, CUDA, TIMEOUT. */
 MCLBM_API int mclbm_grad_required_bytes(const mclbm_ctx* ctx, int64_t nsteps, int32_t ckpt_every, size_t* bytes);
 MCLBM_API int mclbm_grad(mclbm_ctx* ctx, int32_t objective, int64_t nsteps, int32_t ckpt_every, void* d_buf,
                          size_t buf_bytes, double* J, double* dJdX);
@@ -401,8 +406,9 @@ MCLBM_API int mclbm_grad_timing(const mclbm_ctx* ctx, double* ms);
 MCLBM_API int mclbm_adjoint_step(const mclbm_ctx* ctx, const double* d_f, const double* d_lambda_next, double* d_lambda);
 
 /* Synchronise the context's stream and report a bounded device wait that gave up
- * since the last initialisation (MCLBM_ERR_TIMEOUT; the staged stepper's producer and
- * consumer waits are bounded and set this instead of hanging). */
+ * since the last initialisation or load (MCLBM_ERR_TIMEOUT; the waits of the multi-step kernel, for
+ * the tiles of the step before, and of the staged kernel's producer and consumers are bounded and set this
+ * instead of hanging). */
 MCLBM_API int mclbm_device_status(mclbm_ctx* ctx);
 
 /* W_{1,1} on restricted fields like mclbm_w1_restricted, for callers that cannot
@@ -447,7 +453,8 @@ MCLBM_API int mclbm_selftest_timeout(mclbm_ctx* ctx);
  * same lattice (Q), N, M, precision, pattern, options, viscosity, U_c and derived time step,
  * U_lat and omega (anything else would resume the state under other dynamics).
  * Errors: IO (cannot open, truncated, another format version, bytes after the lattice, not
- * a checkpoint), SHAPE (another lattice or configuration), CUDA. */
+ * a checkpoint), SHAPE (another lattice or configuration), TIMEOUT (mclbm_save: steps are missing from the
+ * state, no file is written), CUDA. */
 MCLBM_API int mclbm_save(const mclbm_ctx* ctx, const char* path);
 MCLBM_API int mclbm_load(mclbm_ctx* ctx, const char* path);
 

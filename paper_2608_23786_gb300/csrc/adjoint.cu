@@ -734,7 +734,7 @@ int run_grad(mclbm_ctx* c, int objective, int64_t nsteps, int K, char* buf, size
     MCLBM_CUDA(e);
     pe.mark(5, c->stream);
     MCLBM_CUDA(cudaMemcpyAsync(h_dJdX, out, sizeof(double) * 24 * c->M, cudaMemcpyDeviceToHost, c->stream));
-    MCLBM_CUDA(cudaStreamSynchronize(c->stream));
+    MCLBM_CUDA(read_status(c));
     // with the Leray option the kernels differentiate with respect to the evaluated
     // coefficients Y = L X; dJ/dX = L^T dJ/dY
     if (c->cfg.options & MCLBM_OPT_LERAY) leray_map(h_dJdX, c->M, true, h_dJdX);
@@ -747,7 +747,7 @@ int run_grad(mclbm_ctx* c, int objective, int64_t nsteps, int K, char* buf, size
         c->grad_ms[2] = adjoint_ms;
         c->grad_ms[3] = p;
     }
-    return MCLBM_OK;
+    return waits_held(c);
 }
 
 // One adjoint step on caller data (natural layouts): state f^t [M][19][n] FP64 raw populations,

@@ -200,6 +200,14 @@ int set_error(int code, const std::string& msg)
     return code;
 }
 
+int waits_held(int status)
+{
+    if (status != MCLBM_ERR_TIMEOUT) return MCLBM_OK;
+    return set_error(MCLBM_ERR_TIMEOUT, "a bounded device wait of the stepper gave up: steps are missing from the state "
+                                        "until the next initialisation or load");
+}
+int waits_held(const mclbm_ctx* c) { return waits_held(c->wait_status); }
+
 int cuda_check(cudaError_t e, const char* what)
 {
     return set_error(MCLBM_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
@@ -218,7 +226,6 @@ WorkLayout work_layout(int N, int M)
     wl.params = take((size_t)M * 24 * sizeof(double));
     size_t part = (size_t)M * 2 * 1024 * sizeof(double);
     wl.partial = take(part > kPartialBytes ? part : kPartialBytes);
-    wl.flag = take(16 * sizeof(int));
     wl.field = take(4 * n * sizeof(double));
     wl.cplx = take(n * 2 * sizeof(double));
     const size_t sfb = sf_axes_partial_bytes(N);
@@ -228,10 +235,29 @@ WorkLayout work_layout(int N, int M)
     wl.trig = take((size_t)N * 4 * (sizeof(double) + sizeof(float)));  // FP64 table, then its FP32 copy
     size_t per = 2 * (size_t)(N / 2 + 1);
     if ((size_t)7 * (N / 2) > per) per = (size_t)7 * (N / 2);
+    wl.flag = take(16 * sizeof(int));
     wl.bins = take((size_t)M * per * sizeof(double) + 2 * (size_t)M * sizeof(double));
     wl.total = off;
     return wl;
 }
+
+cudaError_t read_results(mclbm_ctx* c, size_t count, const double** out)
+{
+    const size_t lead = c->wl.bins - c->wl.flag, bytes = lead + count * sizeof(double);
+    try {
+        if (c->staging.size() < bytes) c->staging.resize(bytes);
+    } catch (const std::exception&) {
+        return cudaErrorMemoryAllocation;
+    }
+    cudaError_t e = cudaMemcpyAsync(c->staging.data(), c->work + c->wl.flag, bytes, cudaMemcpyDeviceToHost, c->stream);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return e;
+    std::memcpy(&c->wait_status, c->staging.data() + sizeof(int), sizeof(int));
+    if (out) *out = reinterpret_cast<const double*>(c->staging.data() + lead);
+    return cudaSuccess;
+}
+
+cudaError_t read_status(mclbm_ctx* c) { return read_results(c, 0, nullptr); }
 
 void* lattice_ptr(const mclbm_ctx* c, int which)
 {
@@ -337,6 +363,7 @@ int mclbm_create(const mclbm_config* cfg, void* d_pop, size_t pop_bytes, void* d
     if (cfg->precision == MCLBM_FP64 && c->launch.kind == 0 && (int64_t)cfg->M * c->n <= (1 << 20))
         c->launch.vec = c->launch_odd.vec = 1;
     c->launch_chosen = false;
+    c->wait_status = 0;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
     c->num_sms = sms;
@@ -455,7 +482,7 @@ int mclbm_energy(mclbm_ctx* ctx, double* E, double* Z)
     if (!ctx || !E) return set_error(MCLBM_ERR_INVALID_ARG, "bad argument");
     MCLBM_ON_DEVICE(ctx->device);
     MCLBM_CUDA(launch_energy(ctx, Z != nullptr, E, Z));
-    return MCLBM_OK;
+    return waits_held(ctx);
 }
 
 int mclbm_mean_var(mclbm_ctx* ctx, double* d_mean, double* d_var)
@@ -475,10 +502,10 @@ int mclbm_energy_mean_var(mclbm_ctx* ctx, double* E, double* d_mean, double* d_v
     if (ctx->M > 1024) {  // the one-pass kernel reduces up to 1024 energies in shared memory
         MCLBM_CUDA(launch_mean_var(ctx, d_mean, d_var));
         MCLBM_CUDA(launch_energy(ctx, false, E, nullptr));
-        return MCLBM_OK;
+        return waits_held(ctx);
     }
     MCLBM_CUDA(launch_energy_mean_var(ctx, E, d_mean, d_var));
-    return MCLBM_OK;
+    return waits_held(ctx);
 }
 
 static int ensure_twiddles(mclbm_ctx* ctx)
@@ -497,7 +524,7 @@ int mclbm_spectrum(mclbm_ctx* ctx, double* E)
     int st = ensure_twiddles(ctx);
     if (st != MCLBM_OK) return st;
     MCLBM_CUDA(launch_spectral(ctx, E, nullptr));
-    return MCLBM_OK;
+    return waits_held(ctx);
 }
 
 int mclbm_sf_trace(mclbm_ctx* ctx, double* S2)
@@ -507,7 +534,7 @@ int mclbm_sf_trace(mclbm_ctx* ctx, double* S2)
     int st = ensure_twiddles(ctx);
     if (st != MCLBM_OK) return st;
     MCLBM_CUDA(launch_spectral(ctx, nullptr, S2));
-    return MCLBM_OK;
+    return waits_held(ctx);
 }
 
 int mclbm_sf_axes(mclbm_ctx* ctx, int32_t pmax, double* S)
@@ -516,7 +543,7 @@ int mclbm_sf_axes(mclbm_ctx* ctx, int32_t pmax, double* S)
     MCLBM_ON_DEVICE(ctx->device);
     if (ctx->N > 512) return set_error(MCLBM_ERR_SHAPE, "axis structure functions support N <= 512");
     MCLBM_CUDA(launch_sf_axes(ctx, pmax, S));
-    return MCLBM_OK;
+    return waits_held(ctx);
 }
 
 int mclbm_restrict(const mclbm_ctx* ctx, int32_t Qd, double* d_out)
@@ -561,7 +588,17 @@ int mclbm_w1_1pt(mclbm_ctx* A, const mclbm_ctx* B, int32_t Qd, double* W, double
     Bv.stream = A->stream;
     MCLBM_CUDA(launch_restrict(A, Qd, ra));
     MCLBM_CUDA(launch_restrict(&Bv, Qd, rb));
-    MCLBM_CUDA(launch_w1(ra, A->M, rb, B->M, G, scratch, w1_work_bytes(A->M, B->M, G), A->stream, W, per_point));
+    const int* err_a = (const int*)(A->work + A->wl.flag) + 1;
+    const int* err_b = (const int*)(B->work + B->wl.flag) + 1;
+    MCLBM_CUDA(launch_w1(ra, A->M, rb, B->M, G, scratch, w1_work_bytes(A->M, B->M, G), A->stream, W, per_point, err_a, err_b));
+    if (std::isnan(*W)) {  // NaN fields, or an error word is set: look which
+        int h[2] = {0, 0};
+        MCLBM_CUDA(cudaMemcpyAsync(&h[0], err_a, sizeof(int), cudaMemcpyDeviceToHost, A->stream));
+        MCLBM_CUDA(cudaMemcpyAsync(&h[1], err_b, sizeof(int), cudaMemcpyDeviceToHost, A->stream));
+        MCLBM_CUDA(cudaStreamSynchronize(A->stream));
+        for (const int status : h)
+            if (const int st = waits_held(status)) return st;
+    }
     return MCLBM_OK;
 }
 
@@ -569,12 +606,8 @@ int mclbm_device_status(mclbm_ctx* ctx)
 {
     if (!ctx) return set_error(MCLBM_ERR_INVALID_ARG, "ctx is NULL");
     MCLBM_ON_DEVICE(ctx->device);
-    int flags[2] = {0, 0};
-    MCLBM_CUDA(cudaMemcpyAsync(flags, ctx->work + ctx->wl.flag, sizeof(flags), cudaMemcpyDeviceToHost, ctx->stream));
-    MCLBM_CUDA(cudaStreamSynchronize(ctx->stream));
-    if (flags[1] == MCLBM_ERR_TIMEOUT)
-        return set_error(MCLBM_ERR_TIMEOUT, "a bounded device wait of the staged stepper gave up");
-    return MCLBM_OK;
+    MCLBM_CUDA(read_status(ctx));
+    return waits_held(ctx);
 }
 
 int mclbm_selftest_timeout(mclbm_ctx* ctx)
@@ -612,8 +645,12 @@ int mclbm_save(const mclbm_ctx* ctx, const char* path)
     MCLBM_ON_DEVICE(ctx->device);
     const size_t bytes = ctx->elem_bytes * Q * (size_t)ctx->n * ctx->M;
     std::vector<char> host(bytes);
+    int status = 0;
     MCLBM_CUDA(cudaMemcpyAsync(host.data(), lattice_ptr(ctx, ctx->cur), bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    MCLBM_CUDA(cudaMemcpyAsync(&status, (const int*)(ctx->work + ctx->wl.flag) + 1, sizeof(int), cudaMemcpyDeviceToHost,
+                               ctx->stream));
     MCLBM_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (const int st = waits_held(status)) return st;  // no file of a state that was not reached
     FILE* fp = std::fopen(path, "wb");
     if (!fp) return set_error(MCLBM_ERR_IO, std::string("cannot open ") + path + " for writing");
     const uint64_t magic = kMagic, steps = (uint64_t)ctx->steps;
@@ -688,7 +725,7 @@ int mclbm_check_finite(mclbm_ctx* ctx)
     int bad = 0;
     MCLBM_CUDA(launch_check_finite(ctx, &bad));
     if (bad) return set_error(MCLBM_ERR_NONFINITE, "non-finite population found");
-    return MCLBM_OK;
+    return waits_held(ctx);
 }
 
 }  // extern "C"

@@ -6,6 +6,9 @@
 // so results are bitwise reproducible from run to run (no floating-point atomics).
 #include <cuda_fp16.h>
 
+#include <algorithm>
+#include <cstring>
+
 #include "internal.h"
 #include "stepper_impl.cuh"
 #include "storage.cuh"
@@ -429,13 +432,11 @@ cudaError_t energy_t(mclbm_ctx* c, bool with_z, double* h_E, double* h_Z)
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(h_E, res, sizeof(double) * c->M, cudaMemcpyDeviceToHost, c->stream);
-    if (e != cudaSuccess) return e;
-    if (with_z) {
-        e = cudaMemcpyAsync(h_Z, res + c->M, sizeof(double) * c->M, cudaMemcpyDeviceToHost, c->stream);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaStreamSynchronize(c->stream);
+    const double* h = nullptr;
+    if ((e = read_results(c, (with_z ? 2 : 1) * (size_t)c->M, &h)) != cudaSuccess) return e;
+    std::copy(h, h + c->M, h_E);
+    if (with_z) std::copy(h + c->M, h + 2 * (size_t)c->M, h_Z);
+    return cudaSuccess;
 }
 
 // persistent grid of the statistics pass (fixed: deterministic sums)
@@ -443,7 +444,7 @@ template <class E>
 constexpr int kStatsBlocks = 152 * (kRunScalar<E> ? 6 : 4);
 
 template <class E>
-cudaError_t stats_pass_t(const mclbm_ctx* c, double* d_mean, double* d_var, double* h_E)
+cudaError_t stats_pass_t(mclbm_ctx* c, double* d_mean, double* d_var, double* h_E)
 {
     const Geom g = geom_of(c);
     const E* lat = (const E*)lattice_ptr(c, c->cur);
@@ -476,12 +477,14 @@ cudaError_t stats_pass_t(const mclbm_ctx* c, double* d_mean, double* d_var, doub
     if (e != cudaSuccess || !h_E) return e;
     k_reduce_rows<<<c->M, kBlock, 0, c->stream>>>(partial, c->M, (int)blocks, 1, 0, 1.0 / (double)c->n, res);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaMemcpyAsync(h_E, res, sizeof(double) * c->M, cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return e;
-    return cudaStreamSynchronize(c->stream);
+    const double* h = nullptr;
+    if ((e = read_results(c, c->M, &h)) != cudaSuccess) return e;
+    std::copy(h, h + c->M, h_E);
+    return cudaSuccess;
 }
 
 template <class E>
-cudaError_t mean_var_t(const mclbm_ctx* c, double* d_mean, double* d_var)
+cudaError_t mean_var_t(mclbm_ctx* c, double* d_mean, double* d_var)
 {
     return stats_pass_t<E>(c, d_mean, d_var, nullptr);
 }
@@ -503,8 +506,9 @@ cudaError_t finite_t(mclbm_ctx* c, int* h_bad)
     const int64_t count = (int64_t)c->M * Q * c->n;
     k_check_finite<E><<<grid_for(count), kBlock, 0, c->stream>>>((const E*)lattice_ptr(c, c->cur), count, flag);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaMemcpyAsync(h_bad, flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess) return e;
-    return cudaStreamSynchronize(c->stream);
+    if ((e = read_status(c)) != cudaSuccess) return e;
+    std::memcpy(h_bad, c->staging.data(), sizeof(int));
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -524,12 +528,12 @@ cudaError_t launch_energy(mclbm_ctx* c, bool with_z, double* h_E, double* h_Z)
 {
     MCLBM_DISPATCH(c, energy_t, c, with_z, h_E, h_Z);
 }
-cudaError_t launch_energy_mean_var(const mclbm_ctx* c, double* h_E, double* d_mean, double* d_var)
+cudaError_t launch_energy_mean_var(mclbm_ctx* c, double* h_E, double* d_mean, double* d_var)
 {
     MCLBM_DISPATCH(c, stats_pass_t, c, d_mean, d_var, h_E);
 }
 
-cudaError_t launch_mean_var(const mclbm_ctx* c, double* d_mean, double* d_var)
+cudaError_t launch_mean_var(mclbm_ctx* c, double* d_mean, double* d_var)
 {
     MCLBM_DISPATCH(c, mean_var_t, c, d_mean, d_var);
 }

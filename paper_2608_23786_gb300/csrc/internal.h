@@ -16,7 +16,6 @@ namespace mclbm {
 struct WorkLayout {
     size_t params;    // [M][24] double
     size_t partial;   // reduction partials, kPartialBytes
-    size_t flag;      // int status words (16 ints)
     size_t field;     // velocity fields [4][n] double: one sample's [3][n], or during the paired
                       // spectra the second sample's [3][n] below the first one's u_z
     size_t cplx;      // complex FFT buffer [n] double2
@@ -24,7 +23,8 @@ struct WorkLayout {
     size_t real2;     // power spectrum of the second sample of a pair [n] double
     size_t twiddle;   // [N] double2: exp(-2 pi i j / N), j < N
     size_t trig;      // [N][4] double: sin, cos of x_n and 2 x_n; then the same [N][4] as float
-    size_t bins;      // shell sums [2][N/2+1] double x M
+    size_t flag;      // int status words (16 ints), right before the results: one copy brings both
+    size_t bins;      // results: shell sums [2][N/2+1] double x M and the like
     size_t total;
 };
 
@@ -55,6 +55,8 @@ struct mclbm_ctx {
     mclbm::LaunchConfig launch_odd;  // AA odd steps (pull: equal to launch)
     bool launch_chosen;              // the caller set a shape: every step is a launch of that shape
     int num_sms;
+    int wait_status;                  // error word (MCLBM_ERR_TIMEOUT or 0) as the last copy to the host found it
+    std::vector<char> staging;        // that copy
     double grad_ms[4];  // last mclbm_grad: forward, recompute, reverse (adjoint kernels), parameter reduction
 };
 
@@ -63,6 +65,9 @@ namespace mclbm {
 // error reporting (thread-local message)
 int set_error(int code, const std::string& msg);
 int cuda_check(cudaError_t e, const char* what);
+// MCLBM_ERR_TIMEOUT where an error word (or the one that c->wait_status holds) says that a wait gave up.
+int waits_held(int status);
+int waits_held(const mclbm_ctx* c);
 #define MCLBM_CUDA(call)                                           \
     do {                                                           \
         cudaError_t e_ = (call);                                   \
@@ -105,6 +110,12 @@ WorkLayout work_layout(int N, int M);
 // pointers of the population lattices
 void* lattice_ptr(const mclbm_ctx* c, int which);
 
+// The first `count` doubles of the results region and the status words before it, in one copy; waits
+// for the stream and notes the error word in c->wait_status.  *out: the doubles, valid until the next call.
+cudaError_t read_results(mclbm_ctx* c, size_t count, const double** out);
+// The status words alone.
+cudaError_t read_status(mclbm_ctx* c);
+
 // kernels (launchers return cudaError_t of the launch)
 cudaError_t launch_init(const mclbm_ctx* c, const double* d_params);
 cudaError_t launch_step(mclbm_ctx* c);  // one step of one context; updates cur and steps
@@ -129,15 +140,16 @@ cudaError_t launch_set_populations(mclbm_ctx* c, int sample, const double* d_in)
 cudaError_t launch_moments(const mclbm_ctx* c, int sample, double* d_rho, double* d_u);
 cudaError_t launch_field(const mclbm_ctx* c, int sample, double* d_u);  // physical u [3][n]
 cudaError_t launch_energy(mclbm_ctx* c, bool with_enstrophy, double* h_E, double* h_Z);
-cudaError_t launch_mean_var(const mclbm_ctx* c, double* d_mean, double* d_var);
+cudaError_t launch_mean_var(mclbm_ctx* c, double* d_mean, double* d_var);
 // mean/var fields and E_m in one pass over the populations (M <= 1024)
-cudaError_t launch_energy_mean_var(const mclbm_ctx* c, double* h_E, double* d_mean, double* d_var);
+cudaError_t launch_energy_mean_var(mclbm_ctx* c, double* h_E, double* d_mean, double* d_var);
 cudaError_t launch_restrict(const mclbm_ctx* c, int Q, double* d_out);
 cudaError_t launch_check_finite(mclbm_ctx* c, int* h_bad);
 cudaError_t launch_spectral(mclbm_ctx* c, double* h_E, double* h_S2);
 cudaError_t launch_sf_axes(mclbm_ctx* c, int pmax, double* h_S);
 cudaError_t launch_w1(const double* d_a, int MA, const double* d_b, int MB, int G, char* work, size_t work_bytes,
-                      cudaStream_t s, double* h_W, double* h_per_point);
+                      cudaStream_t s, double* h_W, double* h_per_point, const int* err_a = nullptr,
+                      const int* err_b = nullptr);
 size_t w1_work_bytes(int MA, int MB, int G);
 
 }  // namespace mclbm

@@ -10,6 +10,8 @@
 // keeping its sums in registers across all batches of
 // lines the block handles.  Threads with the same lag are then summed in a fixed
 // order, and a second kernel sums the blocks in a fixed order: deterministic.
+#include <algorithm>
+
 #include "internal.h"
 #include "storage.cuh"
 
@@ -253,10 +255,11 @@ cudaError_t launch_sf_axes(mclbm_ctx* c, int pmax, double* h_S)
                                                out + (int64_t)m * (pmax - 1) * halfN);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = cudaMemcpyAsync(h_S, out, sizeof(double) * c->M * (pmax - 1) * halfN, cudaMemcpyDeviceToHost, c->stream)) !=
-        cudaSuccess)
-        return e;
-    return cudaStreamSynchronize(c->stream);
+    const size_t count = (size_t)c->M * (pmax - 1) * halfN;
+    const double* h = nullptr;
+    if ((e = read_results(c, count, &h)) != cudaSuccess) return e;
+    std::copy(h, h + count, h_S);
+    return cudaSuccess;
 }
 
 }  // namespace mclbm

@@ -19,6 +19,8 @@
 // points {k in K_N : round(|k|) = kappa}, K_N = {-N/2+1..N/2}^3, with an exact
 // integer test 4|k|^2 in [(2 kappa - 1)^2, (2 kappa + 1)^2), each thread over a
 // fixed subset of (k_z, k_y) rows, then fixed reduction trees: deterministic.
+#include <algorithm>
+
 #include "internal.h"
 #include "storage.cuh"
 
@@ -412,12 +414,12 @@ cudaError_t launch_spectral(mclbm_ctx* c, double* h_E, double* h_S2)
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if (h_E && (e = cudaMemcpyAsync(h_E, bins, sizeof(double) * c->M * nb, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-        return e;
-    if (h_S2 && (e = cudaMemcpyAsync(h_S2, bins + (int64_t)c->M * nb, sizeof(double) * c->M * nb, cudaMemcpyDeviceToHost,
-                                     st)) != cudaSuccess)
-        return e;
-    return cudaStreamSynchronize(st);
+    const size_t count = (size_t)c->M * nb;
+    const double* h = nullptr;
+    if ((e = read_results(c, h_S2 ? 2 * count : count, &h)) != cudaSuccess) return e;
+    if (h_E) std::copy(h, h + count, h_E);
+    if (h_S2) std::copy(h + count, h + 2 * count, h_S2);
+    return cudaSuccess;
 }
 
 }  // namespace mclbm

@@ -9,6 +9,8 @@
 // the two sorted lists, accumulating |F_A - F_B| times the gap to the next
 // support point, in FP64.  A final fixed-order reduction gives
 // W = (1/G) sum_points sum_components W1.
+#include <math_constants.h>
+
 #include <cfloat>
 #include <mutex>
 #include <string>
@@ -71,7 +73,9 @@ __global__ void __launch_bounds__(kThreads) k_w1_points(const double* __restrict
     }
 }
 
-__global__ void k_w1_total(const double* __restrict__ per_point, int G, double* __restrict__ out)
+// err_a, err_b: error words of the contexts that the fields come from (or null); a set one makes the total NaN.
+__global__ void k_w1_total(const double* __restrict__ per_point, int G, const int* err_a, const int* err_b,
+                           double* __restrict__ out)
 {
     __shared__ double sh[kThreads];
     double s = 0.0;
@@ -82,7 +86,7 @@ __global__ void k_w1_total(const double* __restrict__ per_point, int G, double* 
         if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[0] = sh[0] / G;
+    if (threadIdx.x == 0) out[0] = (err_a && *err_a) || (err_b && *err_b) ? CUDART_NAN : sh[0] / G;
 }
 
 int pow2_at_least(int v)
@@ -102,7 +106,7 @@ size_t w1_work_bytes(int MA, int MB, int G)
 }
 
 cudaError_t launch_w1(const double* d_a, int MA, const double* d_b, int MB, int G, char* work, size_t work_bytes,
-                      cudaStream_t s, double* h_W, double* h_per_point)
+                      cudaStream_t s, double* h_W, double* h_per_point, const int* err_a, const int* err_b)
 {
     if (work_bytes < w1_work_bytes(MA, MB, G)) return cudaErrorInvalidValue;
     double* per_point = (double*)work;
@@ -112,7 +116,7 @@ cudaError_t launch_w1(const double* d_a, int MA, const double* d_b, int MB, int 
     cudaError_t e = cudaFuncSetAttribute(k_w1_points, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_w1_points<<<dim3(G, 3), kThreads, smem, s>>>(d_a, MA, d_b, MB, G, PA, PB, per_point);
-    k_w1_total<<<1, kThreads, 0, s>>>(per_point, G, total);
+    k_w1_total<<<1, kThreads, 0, s>>>(per_point, G, err_a, err_b, total);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = cudaMemcpyAsync(h_W, total, sizeof(double), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     if (h_per_point &&
@@ -179,7 +183,7 @@ extern "C" int mclbm_w1_restricted_noalloc(const double* d_a, int32_t MA, const 
     const int PA = pow2_at_least(MA), PB = pow2_at_least(MB);
     const size_t smem = (size_t)(PA + PB) * sizeof(double);  // <= 32 KiB: no opt-in needed
     k_w1_points<<<dim3(G, 3), kThreads, smem, s>>>(d_a, MA, d_b, MB, G, PA, PB, pp);
-    k_w1_total<<<1, kThreads, 0, s>>>(pp, G, total);
+    k_w1_total<<<1, kThreads, 0, s>>>(pp, G, nullptr, nullptr, total);
     MCLBM_CUDA(cudaGetLastError());
     MCLBM_CUDA(cudaMemcpyAsync(W, total, sizeof(double), cudaMemcpyDeviceToHost, s));
     if (per_point) MCLBM_CUDA(cudaMemcpyAsync(per_point, pp, sizeof(double) * 3 * G, cudaMemcpyDeviceToHost, s));
