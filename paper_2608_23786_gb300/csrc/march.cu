@@ -166,7 +166,8 @@ cudaError_t march_t(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t 
             e = launch_march_f32(a, vec, mode, c->num_sms, tiles, c->stream);
         else
             e = launch_march_f16(a, vec, mode, c->num_sms, tiles, c->stream);
-        if (e == cudaErrorCooperativeLaunchTooLarge) {  // part of the GPU only: launch by launch
+        // part of the GPU only, or a build whose registers do not allow the kernel's split: launch by launch
+        if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidConfiguration) {
             cudaGetLastError();
             break;
         }

@@ -98,7 +98,7 @@ struct MarchWalk {
 };
 
 template <class E>
-__device__ __forceinline__ MarchWalk march_begin(const MarchArgs<E>& a, unsigned first, unsigned stride)
+__host__ __device__ __forceinline__ MarchWalk march_begin(const MarchArgs<E>& a, unsigned first, unsigned stride)
 {
     const unsigned logct = a.logC + a.logT, ct = 1u << logct;
     MarchWalk p;
@@ -114,7 +114,7 @@ __device__ __forceinline__ MarchWalk march_begin(const MarchArgs<E>& a, unsigned
 }
 
 template <class E>
-__device__ __forceinline__ MarchTile march_next(const MarchArgs<E>& a, MarchWalk& p)
+__host__ __device__ __forceinline__ MarchTile march_next(const MarchArgs<E>& a, MarchWalk& p)
 {
     const unsigned logct = a.logC + a.logT;
     const unsigned logP = a.logU - a.logC;  // chunks per sample
