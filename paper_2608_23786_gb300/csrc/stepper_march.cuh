@@ -62,7 +62,10 @@ constexpr int kMarchAhead = 4;                   // tiles handed out beyond the 
 // Pause between two looks of the warps that keep the books: without it they take issue slots from the
 // colliding warps of their partition (pull 64^3 x 64 61.5 -> 62.1 GLUPS, in another build 59.0 -> 62.1).
 constexpr unsigned kMarchNapNs = 64;
-constexpr uint64_t kMarchLimitNs = 1000ull * 1000 * 1000;  // 1 s of %globaltimer time per wait
+// A wait gives up after 1 s of %globaltimer time and this many looks: a launch that was switched out for a
+// second has looked a few times since, one that makes no progress a million times.
+constexpr uint64_t kMarchLimitNs = 1000ull * 1000 * 1000;
+constexpr unsigned kMarchLimitLooks = 1u << 16;
 
 // What a step reads and writes: the AA pattern in place, the same with the slots of opposite velocities
 // exchanged (a pull lattice), or pull from one lattice to the next.
@@ -215,11 +218,12 @@ struct MarchShared {
     int last[kMarchGroups];      // the group's number of tiles, once known (else -1)
 };
 
-// Gives up a wait: true after kMarchLimitNs (recorded in the error word) or once the error word is set.
-__device__ __forceinline__ bool march_give_up(uint64_t t0, int* err)
+// Gives up a wait after `looks` looks since t0: true past both limits (recorded in the error word) or once
+// the error word is set.
+__device__ __forceinline__ bool march_give_up(uint64_t t0, unsigned looks, int* err)
 {
     if (*(volatile const int*)err != 0) return true;
-    if (global_ns() - t0 <= kMarchLimitNs) return false;
+    if (looks < kMarchLimitLooks || global_ns() - t0 <= kMarchLimitNs) return false;
     atomicExch(err, kTimeoutCode);
     return true;
 }
@@ -244,7 +248,7 @@ __device__ __forceinline__ void march_hand_out(const MarchArgs<E>& a, MarchShare
             if (go && t.valid && lane < 3) go = ld_acquire_gpu(c) >= need;
             if (__all_sync(0xffffffffu, go)) break;
             __nanosleep(kMarchNapNs);
-            if ((it & 63) == 0 && __any_sync(0xffffffffu, lane == 0 && march_give_up(t0, a.err))) return;
+            if ((it & 63) == 0 && __any_sync(0xffffffffu, lane == 0 && march_give_up(t0, it, a.err))) return;
         }
         // Lanes 0, 1 and 2 each acquired one counter; a vote orders no memory, so without this lane 0's
         // release would not carry what lanes 1 and 2 acquired.
@@ -269,7 +273,7 @@ __device__ __forceinline__ void march_report(const MarchArgs<E>& a, MarchShared&
         for (unsigned it = 1; !mbar_test(bar + 8 * (n & (kMarchAhead - 1)), (n / kMarchAhead) & 1); ++it) {
             __nanosleep(kMarchNapNs);
             if ((it & 15) == 0 && ld_acquire_cta(smem_u32(&sh.last[g])) == n) return;
-            if ((it & 255) == 0 && march_give_up(t0, a.err)) return;
+            if ((it & 255) == 0 && march_give_up(t0, it, a.err)) return;
         }
         const unsigned ctr = sh.tile[g][n & (2 * kMarchAhead - 1)].ctr;
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
@@ -357,7 +361,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1) k_march(const __grid_constan
                 const uint64_t t0 = global_ns();
                 for (unsigned it = 1; !ok; ++it) {
                     ok = __all_sync(0xffffffffu, ld_acquire_cta(out) > j + 1);
-                    if (!ok && (it & 255) == 0 && __any_sync(0xffffffffu, lane == 0 && march_give_up(t0, a.err))) return;
+                    if (!ok && (it & 255) == 0 && __any_sync(0xffffffffu, lane == 0 && march_give_up(t0, it, a.err))) return;
                 }
             }
             if (ok) {

@@ -9,7 +9,7 @@ SRC = os.path.join(ROOT, "paper_2608_23786_gb300", "csrc", "stepper_march.cuh")
 
 def _body(name):
     text = re.sub(r"//[^\n]*", "", open(SRC).read())
-    start = text.index("{", re.search(rf"\bvoid {name}\(", text).start())
+    start = text.index("{", re.search(rf"\b(?:void|bool) {name}\(", text).start())
     depth = 0
     for k in range(start, len(text)):
         depth += {"{": 1, "}": -1}.get(text[k], 0)
@@ -31,3 +31,11 @@ def test_every_warp_of_a_tile_orders_its_lanes_before_it_arrives():
     body = re.sub(r"//[^\n]*", "", open(SRC).read())
     arrive = body.rindex("mbar_arrive(")
     assert "__syncwarp()" in body[body.rindex("scatter_all", 0, arrive):arrive]
+
+
+def test_a_wait_gives_up_by_time_and_by_looks():
+    """Time alone would take a launch that was switched out for a second for one without progress."""
+    body = _body("march_give_up").replace("\n", " ")
+    assert re.search(r"looks < kMarchLimitLooks \|\| global_ns\(\) - t0 <= kMarchLimitNs\) return false", body)
+    calls = re.findall(r"march_give_up\(([^)]*)\)", re.sub(r"//[^\n]*", "", open(SRC).read()))
+    assert len(calls) == 4 and calls.count("t0, it, a.err") == 3
