@@ -179,6 +179,20 @@ MCLBM_API int mclbm_get_params(const mclbm_ctx* ctx, double* params);
  * Enqueued only.  Errors: INVALID_ARG, CUDA. */
 MCLBM_API int mclbm_step(mclbm_ctx* ctx, int64_t nsteps);
 
+/* Most steps that one launch of the multi-step kernel takes on this context (odd limits above 1 count as
+ * the even number below); 0, the default: about a second's.  1: every step is a launch of its own.  The
+ * results do not depend on it.  A launch holds the multiprocessors it runs on until its last step, so work of
+ * other streams waits for it: contexts on several streams take turns launch by launch.  Several small
+ * ensembles (below about 32^3 x 5) stepped at once on streams of their own leave the GPU less idle with a
+ * limit of 1: four FP32 contexts of 32^3 x 3, 200 steps each in calls of 12, 1.65 ms against 3.2 (one context
+ * alone 1.19 against 0.88); larger ones do not (64^3 x 4: 4.8 ms against 3.5).
+ * Errors: INVALID_ARG (steps < 0). */
+MCLBM_API int mclbm_set_step_limit(mclbm_ctx* ctx, int64_t steps);
+
+/* Launches of the multi-step kernel enqueued on this context so far (by mclbm_step, mclbm_batch_step and
+ * mclbm_grad) and the steps they take; either may be NULL. */
+MCLBM_API int mclbm_get_step_launches(const mclbm_ctx* ctx, int64_t* launches, int64_t* steps);
+
 /* Number of steps taken since the last initialisation. */
 MCLBM_API int64_t mclbm_steps_taken(const mclbm_ctx* ctx);
 

@@ -363,6 +363,7 @@ int mclbm_create(const mclbm_config* cfg, void* d_pop, size_t pop_bytes, void* d
     if (cfg->precision == MCLBM_FP64 && c->launch.kind == 0 && (int64_t)cfg->M * c->n <= (1 << 20))
         c->launch.vec = c->launch_odd.vec = 1;
     c->launch_chosen = false;
+    c->step_limit = c->multi_launches = c->multi_steps = 0;
     c->wait_status = 0;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
@@ -448,6 +449,21 @@ int mclbm_step(mclbm_ctx* ctx, int64_t nsteps)
     int64_t taken = 0;
     MCLBM_CUDA(launch_march(ctx, nsteps, &taken));
     for (int64_t s = taken; s < nsteps; ++s) MCLBM_CUDA(launch_step(ctx));
+    return MCLBM_OK;
+}
+
+int mclbm_set_step_limit(mclbm_ctx* ctx, int64_t steps)
+{
+    if (!ctx || steps < 0) return set_error(MCLBM_ERR_INVALID_ARG, "bad ctx or steps < 0");
+    ctx->step_limit = steps;
+    return MCLBM_OK;
+}
+
+int mclbm_get_step_launches(const mclbm_ctx* ctx, int64_t* launches, int64_t* steps)
+{
+    if (!ctx) return set_error(MCLBM_ERR_INVALID_ARG, "ctx is NULL");
+    if (launches) *launches = ctx->multi_launches;
+    if (steps) *steps = ctx->multi_steps;
     return MCLBM_OK;
 }
 

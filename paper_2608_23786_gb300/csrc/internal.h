@@ -54,6 +54,8 @@ struct mclbm_ctx {
     mclbm::LaunchConfig launch;      // stepper variant of pull steps and AA even steps (autotuned or default)
     mclbm::LaunchConfig launch_odd;  // AA odd steps (pull: equal to launch)
     bool launch_chosen;              // the caller set a shape: every step is a launch of that shape
+    int64_t step_limit;               // most steps of one launch of the multi-step kernel (0: about a second)
+    int64_t multi_launches, multi_steps;  // its launches so far, and the steps they took
     int num_sms;
     int wait_status;                  // error word (MCLBM_ERR_TIMEOUT or 0) as the last copy to the host found it
     std::vector<char> staging;        // that copy

@@ -23,8 +23,17 @@ constexpr int64_t kL2Bytes = int64_t(90) << 20;
 // 64^3 x 64 and 128^3 x 32 FP32: 2.5 to 5 within 2% of each other, 2 with the window's edge in sight.
 constexpr int64_t kDistance2 = 7;  // in halves
 
-// Longest launch: updates after which a launch ends and the next begins (about a second).
-constexpr int64_t kMaxUpdates = int64_t(4) << 33;
+// Longest launch without a limit of the caller: about a second of steps, by the slowest step measured (a
+// floor for the smallest ensembles, FP32 2.6 to 3 us, FP16 2.4 to 3, FP64 13.9; a rate beyond, D3Q27 FP32 42 and
+// FP64 1.2 GLUPS).  The next launch adds 11 us.
+int64_t longest_launch(const mclbm_ctx* c)
+{
+    if (c->step_limit > 0) return c->step_limit;
+    const bool f64 = c->cfg.precision == MCLBM_FP64;
+    const double floor_ns = f64 ? 14000.0 : 3000.0, nodes_ns = (f64 ? 1.0 : 0.03) * (double)c->M * (double)c->n;
+    const double steps = 1e9 / (nodes_ns > floor_ns ? nodes_ns : floor_ns);
+    return steps > 2.0 ? (int64_t)steps : 2;
+}
 
 int ilog2(int64_t v)
 {
@@ -106,7 +115,7 @@ bool march_order(MarchArgs<E>& a, const mclbm_ctx* c, int vec, int64_t steps)
 // 27.2, x 2 49.9 against 41.5, 8^3 15.0 against 15.2.  Rows within one warp only (N <= 32).
 bool march_serves(const mclbm_ctx* c, int64_t steps)
 {
-    if ((c->cfg.options & MCLBM_OPT_EXACT_GAMMA) || c->launch_chosen) return false;
+    if ((c->cfg.options & MCLBM_OPT_EXACT_GAMMA) || c->launch_chosen || c->step_limit == 1) return false;
     const int64_t nodes = (int64_t)c->M * c->n;
     if (c->cfg.precision == MCLBM_FP64) return c->N <= 32 && nodes <= 1 << 19 && steps >= (nodes <= (1 << 15) ? 16 : 8);
     if (c->cfg.precision == MCLBM_FP16) {
@@ -139,8 +148,7 @@ cudaError_t march_t(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t 
     MarchArgs<E> a;
     memset(&a, 0, sizeof(a));
     const int64_t tiles = (int64_t)c->M * c->n / (kMarchGroup * vec);
-    const int64_t updates = (int64_t)c->M * c->n;
-    const int64_t most = (kMaxUpdates / updates > 2 ? kMaxUpdates / updates : 2) & ~(int64_t)1;
+    const int64_t most = longest_launch(c) & ~(int64_t)1;  // even: the next launch begins at the same parity
     while (*taken < nsteps) {
         int64_t k = nsteps - *taken < most ? nsteps - *taken : most;
         if (mode == kMarchSwap) k &= ~(int64_t)1;
@@ -173,6 +181,8 @@ cudaError_t march_t(mclbm_ctx* c, int mode, const void* src, void* dst, int64_t 
         }
         if (e != cudaSuccess) return e;
         *taken += k;
+        c->multi_launches += 1;
+        c->multi_steps += k;
     }
     return cudaSuccess;
 }

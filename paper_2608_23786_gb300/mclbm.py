@@ -68,6 +68,8 @@ _SIGNATURES = {
     "mclbm_get_params": (_c.c_int, [_ctx_p, _dp]),
     "mclbm_step": (_c.c_int, [_ctx_p, _c.c_int64]),
     "mclbm_steps_taken": (_c.c_int64, [_ctx_p]),
+    "mclbm_set_step_limit": (_c.c_int, [_ctx_p, _c.c_int64]),
+    "mclbm_get_step_launches": (_c.c_int, [_ctx_p, _c.POINTER(_c.c_int64), _c.POINTER(_c.c_int64)]),
     "mclbm_get_populations": (_c.c_int, [_ctx_p, _c.c_int32, _vp]),
     "mclbm_set_populations": (_c.c_int, [_ctx_p, _c.c_int32, _vp]),
     "mclbm_moments": (_c.c_int, [_ctx_p, _c.c_int32, _vp, _vp]),
@@ -282,6 +284,17 @@ def mclbm_step(ctx, nsteps):
 
 def mclbm_steps_taken(ctx):
     return _L(ctx).mclbm_steps_taken(ctx)
+
+
+def mclbm_set_step_limit(ctx, steps):
+    _check(_L(ctx).mclbm_set_step_limit(ctx, int(steps)))
+
+
+def mclbm_get_step_launches(ctx):
+    """(launches, steps) of the multi-step kernel on the context so far."""
+    n, k = ctypes.c_int64(), ctypes.c_int64()
+    _check(_L(ctx).mclbm_get_step_launches(ctx, ctypes.byref(n), ctypes.byref(k)))
+    return n.value, k.value
 
 
 def mclbm_get_populations(ctx, sample, d_out):

@@ -81,16 +81,21 @@ static mclbm_ctx context(int N, int M, int precision, int pattern)
 extern "C" {
 
 // Steps taken by the multi-step kernel of a call for nsteps (negative: the CUDA error of the call).
-int64_t take(int N, int M, int precision, int pattern, int64_t nsteps, int answer)
+int64_t take(int N, int M, int precision, int pattern, int64_t nsteps, int answer, int64_t limit, int trajectory)
 {
     g_launches.clear();
     g_answer = (cudaError_t)answer;
     mclbm_ctx c = context(N, M, precision, pattern);
+    c.step_limit = limit;
     int64_t taken = -1;
-    const cudaError_t e = launch_march(&c, nsteps, &taken);
+    const cudaError_t e = trajectory ? launch_march_trajectory(&c, (void*)(kBase / 2), (void*)kBase, c.pop_bytes, nsteps, &taken)
+                                     : launch_march(&c, nsteps, &taken);
     if (e != cudaSuccess) return -(int64_t)e;
-    return c.steps == taken ? taken : -100000;
+    const bool counted = c.multi_launches == (int64_t)g_launches.size() && c.multi_steps == taken;
+    return counted && c.steps == (trajectory ? 0 : taken) ? taken : -100000;
 }
+
+int velocities() { return Q; }
 
 int launches(int64_t* out, int most)  // [][5]: steps, source, destination, parity of the first step, lanes
 {
