@@ -29,7 +29,6 @@
 //    kept in a column-major matrix in the work buffer, one per block in flight.
 #include <math_constants.h>
 
-#include <cfloat>
 #include <cmath>
 #include <string>
 
@@ -42,6 +41,7 @@ namespace {
 constexpr int kPairMaxL = 256;  // largest assignment of the warp kernel (eight columns per lane)
 constexpr int kPairWarps = 4;   // warps (problems in flight) per block
 constexpr long long kInf = 0x3fffffffffffffffLL;
+constexpr double kCostMax = 1.8e19;  // whose square still is a finite FP32 number
 
 struct PairProblem {
     int i, j, c;  // point pair (i <= j) and component (vector problems: c = 0)
@@ -347,19 +347,17 @@ __global__ void __launch_bounds__(32 * kPairWarps) k_w1_match(const double* __re
             __syncwarp();
         }
         // W1 of the problem: mean FP64 cost of the matched pairs; NaN if the search failed or if the plan
-        // holds a pair whose cost is no number in FP32 (qcost_split gives such costs a finite value
+        // holds a pair whose cost is no finite number in FP32 (qcost_split gives such costs a finite value
         // above any other, so they are in a plan only where it cannot do without)
         double s = 0.0;
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
             const int col = lane + 32 * c;
-            if (col < L) {
-                const int r = pcol[col];
-                if (r >= 0) s += cost64<K>(A, B, G, r / ra, col / rb, pb);
-                failed = failed || r < 0 || !(dist2<K>(row[r].x, y[c]) <= FLT_MAX);
+            if (col < L && pcol[col] >= 0) {
+                const double d = cost64<K>(A, B, G, pcol[col] / ra, col / rb, pb);
+                s += d <= kCostMax ? d : CUDART_NAN;
             }
         }
-        failed = __any_sync(0xffffffffu, failed);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
         if (lane == 0) per[prob] = failed ? CUDART_NAN : s / L;
@@ -754,20 +752,22 @@ int gcd_int(int a, int b)
     return a;
 }
 
-// Whether the warp kernel takes the problems (else the block solver).  Unequal counts: the L x L problem
-// has c = (L / MA)(L / MB) times the entries of the MA x MB one, and equal atoms lengthen its searches, which
-// the block solver does not repeat; the warp kernel, for its part, solves seven times as many problems at
-// once and takes longer for one.  Measured warp / block time against c L (1, 36, 378, 2080 and 23,436
-// vector problems): 100, 50 (200) 0.41, 0.48, 0.3, 0.1, -; 24, 36 (432) 0.53, 0.74, 0.42, 0.13, 0.09; 256, 128
-// (512) 1.02, 1.07, 0.5, 0.25, -; 250, 50 (1250) 1.7, 1.7, 0.95, 0.46, 0.27; 100, 40 (2000) 2.4, 2.6, 1.3, 0.6,
-// 0.4; 256, 16 (4096) 2.8, 2.8, 1.4, 0.7, 0.5; 10, 7 (4900) 3.2, 3.4, 2.5, 0.98, 0.73; 12, 11 (17,424) 8.4, 9.5,
-// 5.5, 3.0, 2.0; 16, 15 (57,600) 20, 22, 13, 6.3, -.  Equal counts: below 0.8 throughout.
+// Whether the warp kernel takes the problems (else the block solver).  Unequal counts: the repeated problem has
+// c = (L / MA)(L / MB) times the entries of the MA x MB one, and equal atoms lengthen its searches, where
+// the block solver repeats nothing; the warp kernel, for its part, solves seven times as many problems at
+// once and takes longer for one, the more so the larger L.  Measured warp / block time (vector problems: 1,
+// 36, 378, 2080 and 23,436 of them) against c and c L^2: 100, 50 (2; 2e4) 0.41, 0.48, 0.3, 0.1, -; 24, 36 (6;
+// 3.1e4) 0.53, 0.74, 0.42, 0.13, 0.09; 200, 100 (2; 8e4) 0.77, 0.86, 0.52, 0.24, 0.15; 256, 128 (2; 1.3e5) 1.02,
+// 1.07, 0.5, 0.25, -; 250, 50 (5; 3.1e5) 1.7, 1.7, 0.95, 0.46, 0.27; 100, 40 (10; 4e5) 2.4, 2.6, 1.3, 0.6, 0.4;
+// 256, 16 (16; 1.05e6) 2.8, 2.8, 1.4, 0.7, 0.5; 10, 7 (70; 3.4e5) 3.2, 3.4, 2.5, 0.98, 0.73; 12, 11 (132; 2.3e6)
+// 8.4, 9.5, 5.5, 3.0, 2.0; 16, 15 (240; 1.4e7) 20, 22, 13, 6.3, -.  Equal counts: below 0.8 throughout.
 bool match_serves(int MA, int MB, int64_t L, int64_t nprob)
 {
     if (L > kPairMaxL) return false;
     if (L <= 64 || MA == MB) return true;
-    const int64_t size = L / MA * (L / MB) * L;
-    return size <= 400 || (size <= 5000 && size <= 3 * nprob);
+    const int64_t copies = L / MA * (L / MB), size = copies * L * L;
+    if (copies > 20 && copies > nprob / 30) return false;
+    return size <= 100000 || (size <= 1200000 && size <= 750 * nprob);
 }
 
 }  // namespace

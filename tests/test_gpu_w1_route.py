@@ -31,10 +31,10 @@ def _gpu(ua, ub, vector):
     return W, per.cpu().numpy()
 
 
-# copies x L: 200 (always repeated); 432, 576 and 1600 (from 144, 192 and 534 problems on); 4900 (1634); 17424
-# and 57600 (never)
-@pytest.mark.parametrize("MA,MB", [(50, 100), (24, 36), (48, 32), (20, 16), (10, 7), (12, 11), (16, 15)])
-@pytest.mark.parametrize("G", [1, 5, 35])
+# atoms repeated: always; always; from 171 (20, 16), 300 (64, 96), 534 (100, 40) and 2100 problems on (10, 7);
+# never; never.  15 problems, 45 by components, and 630, 1890 by components; 2145 and 6435.
+@pytest.mark.parametrize("MA,MB", [(50, 100), (24, 36), (20, 16), (64, 96), (100, 40), (10, 7), (12, 11), (16, 15)])
+@pytest.mark.parametrize("G", [1, 5, 35, 65])
 def test_both_routes_against_the_oracle(MA, MB, G):
     ua = gen.uniform(900 + MA, (MA, G, 3))
     ub = gen.uniform(950 + MB, (MB, G, 3)) * 1.2 + 0.05
