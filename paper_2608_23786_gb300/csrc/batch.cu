@@ -27,7 +27,7 @@ struct mclbm_batch {
     mclbm::LaunchConfig launch_odd;  // AA odd steps
     bool use_graph;
     bool warmed;
-    bool launch_chosen;  // the caller set a shape: every sub-step is a launch of that shape
+    bool launch_chosen;  // the caller or the tuner chose a shape: every sub-step is a launch of that shape
     std::map<std::vector<int64_t>, cudaGraphExec_t> graphs;
     int64_t macro_steps;
 };
@@ -39,6 +39,11 @@ int reinit_ctx(mclbm_ctx* c);  // api.cu: re-run the initialisation from the sto
 using namespace mclbm;
 
 namespace {
+
+// The calls for which the tuners time the multi-step kernel: steps of a context, macro steps of a batch
+// (long enough for every rule of march_serves).
+constexpr int64_t kTunedCall = 48, kTunedMacroSteps = 8;
+constexpr int kTunedRuns = 3;
 
 std::vector<int64_t> signature(const mclbm_batch* b)
 {
@@ -85,6 +90,20 @@ bool most_marches(const mclbm_batch* b, int64_t macro_steps)
         if (march_serves_call(b->lev[l], macro_steps * b->sub[l])) served += updates;
     }
     return served >= 0.875 * all;
+}
+
+// macro_steps macro steps, level by level.
+cudaError_t macro_by_level(mclbm_batch* b, int64_t macro_steps)
+{
+    for (size_t l = 0; l < b->lev.size(); ++l) {
+        const int64_t k = macro_steps * b->sub[l];
+        int64_t taken = 0;
+        cudaError_t e = launch_march(b->lev[l], k, &taken);
+        for (; e == cudaSuccess && taken < k; ++taken)
+            e = launch_levels(&b->lev[l], 1, b->launch, b->launch_odd, b->stream, nullptr);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 struct Saved {
@@ -148,6 +167,18 @@ int time_ms(cudaStream_t s, F&& body, double* ms)
     if (e1 != cudaSuccess) return cuda_check(e1, "cudaEventRecord");
     if (e2 != cudaSuccess) return cuda_check(e2, "cudaEventSynchronize");
     *ms = t;
+    return MCLBM_OK;
+}
+
+template <class F>
+int best_ms_of(int runs, cudaStream_t s, F&& body, double* ms)
+{
+    for (int k = 0; k < runs; ++k) {
+        double t = 0;
+        const int st = time_ms(s, body, &t);
+        if (st != MCLBM_OK) return st;
+        if (k == 0 || t < *ms) *ms = t;
+    }
     return MCLBM_OK;
 }
 
@@ -299,6 +330,19 @@ int mclbm_autotune(mclbm_ctx* ctx, int32_t trial_steps, int32_t* kind, int32_t* 
         ctx->launch_odd = bestc[1];
         per_step = (best[0] + best[1]) / 2;
     }
+    // long calls keep to the multi-step kernel where it is faster than the fastest shape
+    ctx->launch_chosen = false;
+    if (march_serves_call(ctx, kTunedCall)) {
+        int64_t taken = 0;
+        MCLBM_CUDA(launch_march(ctx, kTunedCall, &taken));  // warm-up
+        double ms = 0;
+        int st = best_ms_of(kTunedRuns, ctx->stream, [&]() { return launch_march(ctx, kTunedCall, &taken); }, &ms);
+        if (st != MCLBM_OK) return st;
+        if (taken > 0) {
+            ctx->launch_chosen = ms / taken >= per_step;
+            if (ms / taken < per_step) per_step = ms / taken;
+        }
+    }
     int st = reinit_ctx(ctx);
     if (st != MCLBM_OK) return st;
     if (kind) *kind = ctx->launch.kind;
@@ -355,7 +399,7 @@ int mclbm_batch_create(mclbm_ctx* const* levels, int32_t nlev, const int32_t* su
     }
     b->use_graph = b->stream != nullptr;
     b->warmed = false;
-    b->launch_chosen = false;
+    b->launch_chosen = levels[0]->launch_chosen;  // with the shape
     b->macro_steps = 0;
     *out = b;
     return MCLBM_OK;
@@ -424,12 +468,7 @@ int mclbm_batch_step(mclbm_batch* b, int64_t macro_steps)
     if (!b || macro_steps < 0) return set_error(MCLBM_ERR_INVALID_ARG, "bad argument");
     MCLBM_ON_DEVICE(b->lev[0]->device);
     if (macro_steps > 0 && !b->launch_chosen && most_marches(b, macro_steps)) {
-        for (size_t l = 0; l < b->lev.size(); ++l) {
-            const int64_t k = macro_steps * b->sub[l];
-            int64_t taken = 0;
-            MCLBM_CUDA(launch_march(b->lev[l], k, &taken));
-            for (; taken < k; ++taken) MCLBM_CUDA(launch_levels(&b->lev[l], 1, b->launch, b->launch_odd, b->stream, nullptr));
-        }
+        MCLBM_CUDA(macro_by_level(b, macro_steps));
         b->macro_steps += macro_steps;
         return MCLBM_OK;
     }
@@ -514,6 +553,17 @@ int mclbm_batch_autotune(mclbm_batch* b, int32_t trials, int32_t* kind, int32_t*
         }
     b->launch = bestc;
     b->launch_odd = besto;
+    best /= trials;
+    b->launch_chosen = false;
+    const int64_t call = trials > kTunedMacroSteps ? trials : kTunedMacroSteps;
+    if (most_marches(b, call)) {
+        MCLBM_CUDA(macro_by_level(b, call));  // warm-up
+        double ms = 0;
+        int st = best_ms_of(kTunedRuns, b->stream, [&]() { return macro_by_level(b, call); }, &ms);
+        if (st != MCLBM_OK) return st;
+        b->launch_chosen = ms / call >= best;
+        if (ms / call < best) best = ms / call;
+    }
     clear_graphs(b);
     b->warmed = false;
     for (auto* c : b->lev) {
@@ -524,7 +574,7 @@ int mclbm_batch_autotune(mclbm_batch* b, int32_t trials, int32_t* kind, int32_t*
     if (kind) *kind = bestc.kind;
     if (vec) *vec = bestc.vec;
     if (block) *block = bestc.block;
-    if (best_ms) *best_ms = best / trials;
+    if (best_ms) *best_ms = best;
     return MCLBM_OK;
 }
 

@@ -53,7 +53,7 @@ struct mclbm_ctx {
     bool twiddles_ready;  // FFT twiddle table computed in the work buffer
     mclbm::LaunchConfig launch;      // stepper variant of pull steps and AA even steps (autotuned or default)
     mclbm::LaunchConfig launch_odd;  // AA odd steps (pull: equal to launch)
-    bool launch_chosen;              // the caller set a shape: every step is a launch of that shape
+    bool launch_chosen;              // the caller or the tuner chose a shape: every step is a launch of that shape
     int64_t step_limit;               // most steps of one launch of the multi-step kernel (0: about a second)
     int64_t multi_launches, multi_steps;  // its launches so far, and the steps they took
     int num_sms;

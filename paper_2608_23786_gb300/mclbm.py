@@ -426,7 +426,7 @@ def mclbm_get_launch_parity(ctx, parity):
 
 
 def mclbm_autotune(ctx, trial_steps=5):
-    """Returns (kind, vec, block, ms per step) of the fastest shape."""
+    """(kind, vec, block) of the fastest shape, and the ms per step of a long call."""
     k, v, b, ms = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32(), ctypes.c_double()
     _check(_L(ctx).mclbm_autotune(ctx, int(trial_steps), ctypes.byref(k), ctypes.byref(v), ctypes.byref(b),
                                  ctypes.byref(ms)))
@@ -483,7 +483,7 @@ def mclbm_batch_macro_steps(b):
 
 
 def mclbm_batch_autotune(b, trials=2):
-    """Returns (kind, vec, block, ms per macro step) of the fastest shape."""
+    """(kind, vec, block) of the fastest shape, and the ms per macro step of a long call."""
     k, v, blk, ms = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32(), ctypes.c_double()
     _check(_L(b).mclbm_batch_autotune(b, int(trials), ctypes.byref(k), ctypes.byref(v), ctypes.byref(blk),
                                        ctypes.byref(ms)))
