@@ -65,10 +65,19 @@ def stepper_digest():
     return h.hexdigest()[:16]
 
 
-def takes_multi_step(precision, exact_gamma=False, chosen=False):
-    """Whether a long call of the benchmark's large ensembles runs in the multi-step kernel (FP32
-    storage, closed-form gamma, no launch shape set)."""
-    return precision == "fp32" and not exact_gamma and not chosen
+class MultiStepCount:
+    """Launches of the multi-step kernel on a context, and the steps they took, since this object was made."""
+
+    def __init__(self, ctx):
+        from paper_2608_23786_gb300 import mclbm
+        self._get = lambda: mclbm.mclbm_get_step_launches(ctx)
+        self._launches, self._steps = self._get()
+
+    def launches(self):
+        return self._get()[0] - self._launches
+
+    def steps(self):
+        return self._get()[1] - self._steps
 
 
 def measured_peaks():
@@ -212,6 +221,7 @@ def measure_targets(dev, stream, peaks, peak_kind, lattice=19):
         est = _event_time(stream, step, 4) / 4
         n = _timed_steps(stream, step, est)
         n += n % 2  # whole AA step pairs
+        count = MultiStepCount(ens.ctx)
         with ClockSampler(dev.index or 0) as clk:
             sec = _event_time(stream, step, n)
         mclbm.mclbm_device_status(ens.ctx)
@@ -221,7 +231,7 @@ def measure_targets(dev, stream, peaks, peak_kind, lattice=19):
         launch = launch_desc(mclbm.mclbm_get_launch_parity(ens.ctx, 0),
                              mclbm.mclbm_get_launch_parity(ens.ctx, 1) if pat == "aa" else None)
         out[name] = {"glups": lu / sec / 1e9, "ms_per_update": sec / n * 1e3, "steps_timed": n,
-                     "kernel": MULTI_STEP_KERNEL if takes_multi_step(prec) else KERNEL_NAMES[mclbm.mclbm_get_launch(ens.ctx)[0]],
+                     "kernel": MULTI_STEP_KERNEL if count.steps() else KERNEL_NAMES[mclbm.mclbm_get_launch(ens.ctx)[0]],
                      "bytes_per_lu": bpl, "achieved_gbs": ach, "peak_gbs": peaks["hbm_gbs"], "peak_kind": peak_kind,
                      "frac": ach / peaks["hbm_gbs"], "launch": dict(launch, chosen_by="default"),
                      "clocks": clk.summary()}
@@ -236,6 +246,7 @@ def measure_targets(dev, stream, peaks, peak_kind, lattice=19):
         macro(3)
         est = _event_time(stream, macro, 2) / 2
         n = _timed_steps(stream, macro, est, lo=3, hi=200)
+        count = MultiStepCount(levels[-1].ctx)
         with ClockSampler(dev.index or 0) as clk:
             sec = _event_time(stream, macro, n)
         for e in levels:
@@ -248,7 +259,7 @@ def measure_targets(dev, stream, peaks, peak_kind, lattice=19):
         out[f"levels_64x64_128x32_256x8_{prec}_{pat}"] = {
             "glups": lu / sec / 1e9, "ms_per_macro_step": sec / n * 1e3, "macro_steps_timed": n, "substeps": subs,
             "bytes_per_lu": bpl, "achieved_gbs": ach, "peak_gbs": peaks["hbm_gbs"], "peak_kind": peak_kind,
-            "frac": ach / peaks["hbm_gbs"], "launch": dict(launch, chosen_by="default"), "graph": not takes_multi_step(prec),
+            "frac": ach / peaks["hbm_gbs"], "launch": dict(launch, chosen_by="default"), "graph": count.steps() == 0,
             "clocks": clk.summary()}
         mclbm.mclbm_batch_destroy(b)
         del levels
@@ -709,6 +720,7 @@ def run_levels(args, precision):
         mclbm.mclbm_batch_step(b, 1)
     torch.cuda.synchronize()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    count = MultiStepCount(levels[-1].ctx)
     with ClockSampler(0) as clk:
         ev0.record(stream)
         mclbm.mclbm_batch_step(b, args.steps)
@@ -741,9 +753,9 @@ def run_levels(args, precision):
         "data": "synthetic",
         "config": {"workload": f"levels_64x64_128x32_256x8_{precision}_{pattern}", "substeps": subs,
                    "launch": launch_desc(tuned, mclbm.mclbm_batch_get_launch_parity(b, 1) if pattern == "aa" else None),
-                   "graph": not takes_multi_step(precision),
+                   "graph": count.steps() == 0,
                    "l2": "inputs larger than L2"},
-        "roofline": {"kernel": MULTI_STEP_KERNEL if takes_multi_step(precision) else KERNEL_NAMES[tuned[0]], "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
+        "roofline": {"kernel": MULTI_STEP_KERNEL if count.steps() else KERNEL_NAMES[tuned[0]], "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"], "peak_kind": peak_kind, "traffic": None},
         "stats_once_s": stats_s, "w1_consecutive_levels": w1, "w1_2pt_consecutive_levels": w12,
         "spectrum_finite": bool(all(np.all(np.isfinite(x)) for x in spectra + sfa)),
@@ -967,10 +979,6 @@ def main():
     mean = torch.empty((3,) + (wl["N"],) * 3, dtype=torch.float64, device=dev)
     var = torch.empty_like(mean)
     E = np.zeros(wl["M"])
-    multi = takes_multi_step(wl["precision"], args.exact_gamma, bool(args.launch)) and S >= 12
-    # pull ensembles take an even number of updates in the multi-step kernel
-    stepper_launches = (1 + (S % 2 if wl["pattern"] == "pull" else 0)) if multi else S
-    kernels_per_step = stepper_launches + 2  # and one pass for E(t) and the mean/var fields, its energy reduce
 
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
 
@@ -988,6 +996,7 @@ def main():
     if world > 1:
         dist.barrier()
     torch.cuda.synchronize()
+    count = MultiStepCount(ens.ctx)
     t_start = torch.cuda.Event(enable_timing=True)
     t_end = torch.cuda.Event(enable_timing=True)
     with ClockSampler(local) as clk:
@@ -1000,6 +1009,10 @@ def main():
         dist.barrier()
     torch.cuda.synchronize()
     elapsed = t_start.elapsed_time(t_end) / 1e3
+    multi = count.steps() > 0
+    # launches of the multi-step kernel, and of the updates that are a launch each
+    stepper_launches = (count.launches() + args.steps * S - count.steps()) // args.steps
+    kernels_per_step = stepper_launches + 2  # and one pass for E(t) and the mean/var fields, its energy reduce
     stepper_s = sum(a.elapsed_time(b) for a, b in ev) / 1e3 / (args.steps * S)  # per update of the ensemble
     if world > 1:
         t = torch.tensor([elapsed], dtype=torch.float64)
