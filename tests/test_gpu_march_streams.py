@@ -52,3 +52,26 @@ def test_contexts_on_streams_of_their_own(calls):
         mclbm.mclbm_device_status(got.ctx)
         assert mclbm.mclbm_get_step_launches(got.ctx)[0] == calls
         assert all(torch.equal(got.populations(m), ref.populations(m)) for m in range(ref.M))
+
+
+@pytest.mark.parametrize("precision,N,M,pattern", [("fp32", 32, 7, "pull"), ("fp32", 64, 9, "aa"), ("fp16", 32, 2, "aa"),
+                                                   ("fp64", 32, 2, "pull")])
+def test_a_captured_call_replays(precision, N, M, pattern):
+    """A call of an even number of steps inside a CUDA graph capture, replayed: the bits of the same steps
+    taken one at a time."""
+    stream = torch.cuda.Stream()
+    e = Ensemble(N, M, Re=12.5 * N, Ma=1.6 / 64, precision=precision, pattern=pattern, stream=stream).init()
+    e.step(20)
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        e.step(20)
+    assert mclbm.mclbm_get_step_launches(e.ctx) == (2, 40)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    mclbm.mclbm_device_status(e.ctx)
+    ref = Ensemble(N, M, Re=12.5 * N, Ma=1.6 / 64, precision=precision, pattern=pattern).init()
+    mclbm.mclbm_set_step_limit(ref.ctx, 1)
+    ref.step(80)
+    assert all(torch.equal(e.populations(m), ref.populations(m)) for m in range(M))
