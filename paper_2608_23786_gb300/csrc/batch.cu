@@ -11,11 +11,13 @@
 // to its start) are captured once into a CUDA graph and replayed.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <map>
 #include <string>
 #include <vector>
 
 #include "internal.h"
+#include "lattice.cuh"
 
 struct mclbm_batch {
     std::vector<mclbm_ctx*> lev;
@@ -75,21 +77,66 @@ cudaError_t macro_direct(mclbm_batch* b, const LaunchConfig& cfg, const LaunchCo
     return cudaSuccess;
 }
 
-// The levels are independent, so each can take its steps of a call by itself.  That is the faster way
-// where the multi-step kernel serves the levels that hold the work (at least 7/8 of the updates; the
-// others take too few steps for it, and theirs are single launches).  One macro step, in the sub-steps'
-// launches -> level by level: FP32 16^3 x 4, 32^3 x 2, 64^3 x 2 AA 0.28 -> 0.19 ms, 32^3 x 4, 64^3 x 2,
-// 128^3 x 2 pull 1.68 -> 1.19, 64^3 x 64, 128^3 x 32, 256^3 x 8 56.7 -> 49.2; FP16 AA, six macro steps,
-// 16^3 x 32, 32^3 x 16, 64^3 x 4 1.83 -> 1.73.
-bool most_marches(const mclbm_batch* b, int64_t macro_steps)
+// The levels are independent, so each can take its steps of a call by itself, in the multi-step kernel where
+// that serves it.  Then nothing of one level overlaps another: small levels, which one launch per
+// sub-step covers together, lose what the kernel gains (8^3, 16^3, 32^3 x 1 FP32 pull, two macro steps: 45 us per
+// macro step in sub-steps' launches, 71 level by level).  So both ways are estimated, in microseconds per
+// launch or step, from measurements of three-level batches (levels N, 2N, 4N, one, four and sixteen
+// sub-steps) and of single contexts:
+//   a launch for n thousand nodes in a graph: FP32 2.3 + 0.019 n or 1.5 + 0.0229 n, whichever is more, AA 1.1
+//     more; FP16 4.5 + 0.003 n or 2.6 + 0.0137 n, AA 5.4 + 0.003 n or 3.3 + 0.014 n; FP64 14 or 0.99 n; 1.7 more
+//     without a graph;
+//   a step of the multi-step kernel: FP32 2.7 + 0.0095 n or 0.0172 n; FP16 2.6 + 0.0078 n or 0.0152 n; FP64 14 or
+//     4 + 0.6 n; 11 per call
+// (D3Q27: slopes 27/19), within 12% of the 66 batches measured.  Sub-steps' launches -> level by level, us per macro step: FP32 pull, two macro steps,
+// 16^3 x 4 + 32^3 x 2 + 64^3 123 -> 118, 32^3 x 4 + 64^3 x 2 + 128^3 870 -> 602; AA 146 -> 118, 883 -> 589; FP16 AA 114
+// -> 108, pull 103 -> 108 (stays); FP64 8^3, 16^3, 32^3 560 -> 501; FP32 64^3 x 64 + 128^3 x 32 + 256^3 x 8 56.7 ->
+// 49.2 ms.
+double launch_us(const mclbm_batch* b, double nodes, bool graph)
 {
-    double all = 0, served = 0;
-    for (size_t l = 0; l < b->lev.size(); ++l) {
-        const double updates = (double)b->lev[l]->M * b->lev[l]->n * b->sub[l];
-        all += updates;
-        if (march_serves_call(b->lev[l], macro_steps * b->sub[l])) served += updates;
+    const double kn = nodes * Q / 19.0 / 1000.0;
+    const bool aa = b->lev[0]->cfg.pattern == MCLBM_AA;
+    const double direct = graph ? 0.0 : 1.7;
+    switch (b->lev[0]->cfg.precision) {
+        case MCLBM_FP64: return direct + std::max(14.0, 0.99 * kn);
+        case MCLBM_FP32: return direct + (aa ? 1.1 : 0.0) + std::max(2.3 + 0.019 * kn, 1.5 + 0.0229 * kn);
+        default:
+            return direct + (aa ? std::max(5.4 + 0.003 * kn, 3.3 + 0.014 * kn) : std::max(4.5 + 0.003 * kn, 2.6 + 0.0137 * kn));
     }
-    return served >= 0.875 * all;
+}
+
+double march_us(int precision, double nodes)
+{
+    const double kn = nodes * Q / 19.0 / 1000.0;
+    switch (precision) {
+        case MCLBM_FP64: return std::max(14.0, 4.0 + 0.6 * kn);
+        case MCLBM_FP32: return std::max(2.7 + 0.0095 * kn, 0.0172 * kn);
+        default: return std::max(2.6 + 0.0078 * kn, 0.0152 * kn);
+    }
+}
+
+bool by_level(const mclbm_batch* b, int64_t macro_steps)
+{
+    const bool graph = b->use_graph && macro_steps >= b->period;
+    double levels = 0, together = 0;  // microseconds of a macro step
+    bool any = false;
+    for (size_t l = 0; l < b->lev.size(); ++l) {
+        const double nodes = (double)b->lev[l]->M * (double)b->lev[l]->n;
+        if (march_serves_call(b->lev[l], macro_steps * b->sub[l])) {
+            any = true;
+            levels += 11.0 / (double)macro_steps + b->sub[l] * march_us(b->lev[l]->cfg.precision, nodes);
+        } else {
+            levels += b->sub[l] * launch_us(b, nodes, false);
+        }
+    }
+    if (!any) return false;
+    for (int s = 0; s < b->S; ++s) {
+        double nodes = 0;
+        for (size_t l = 0; l < b->lev.size(); ++l)
+            if (s % (b->S / b->sub[l]) == 0) nodes += (double)b->lev[l]->M * (double)b->lev[l]->n;
+        if (nodes > 0) together += launch_us(b, nodes, graph);
+    }
+    return levels < together;
 }
 
 // macro_steps macro steps, level by level.
@@ -467,7 +514,7 @@ int mclbm_batch_step(mclbm_batch* b, int64_t macro_steps)
 {
     if (!b || macro_steps < 0) return set_error(MCLBM_ERR_INVALID_ARG, "bad argument");
     MCLBM_ON_DEVICE(b->lev[0]->device);
-    if (macro_steps > 0 && !b->launch_chosen && most_marches(b, macro_steps)) {
+    if (macro_steps > 0 && !b->launch_chosen && by_level(b, macro_steps)) {
         MCLBM_CUDA(macro_by_level(b, macro_steps));
         b->macro_steps += macro_steps;
         return MCLBM_OK;
@@ -556,7 +603,7 @@ int mclbm_batch_autotune(mclbm_batch* b, int32_t trials, int32_t* kind, int32_t*
     best /= trials;
     b->launch_chosen = false;
     const int64_t call = trials > kTunedMacroSteps ? trials : kTunedMacroSteps;
-    if (most_marches(b, call)) {
+    if (by_level(b, call)) {
         MCLBM_CUDA(macro_by_level(b, call));  // warm-up
         double ms = 0;
         int st = best_ms_of(kTunedRuns, b->stream, [&]() { return macro_by_level(b, call); }, &ms);

@@ -114,3 +114,24 @@ def test_fp64_batch_level_by_level_equals_single_steps(pattern):
             _same(x, y)
     finally:
         mclbm.mclbm_batch_destroy(b)
+
+
+@pytest.mark.parametrize("pattern", ["pull", "aa"])
+@pytest.mark.parametrize("precision,M,by_level", [("fp32", 1, False), ("fp32", 64, True), ("fp64", 4, True)])
+def test_small_levels_keep_a_launch_per_sub_step(precision, M, by_level, pattern):
+    """Levels too small to be worth a launch of their own (8^3, 16^3, 32^3 of one sample, FP32) stay in one
+    launch per sub-step; either way the levels end in the bits of single steps."""
+    stream = torch.cuda.Stream()
+    pairs = [[Ensemble(8 << k, M, Re=100.0 * 4**k, Ma=0.05 / 2**k, precision=precision, pattern=pattern, stream=stream).init()
+              for _ in range(2)] for k in range(3)]
+    b = mclbm.mclbm_batch_create([a.ctx for a, _ in pairs], [1, 4, 16])
+    try:
+        for _ in range(2):
+            mclbm.mclbm_batch_step(b, 2)
+        assert (mclbm.mclbm_get_step_launches(pairs[2][0].ctx)[0] > 0) == by_level
+        for (x, y), sub in zip(pairs, (1, 4, 16)):
+            for _ in range(4 * sub):
+                y.step(1)
+            _same(x, y)
+    finally:
+        mclbm.mclbm_batch_destroy(b)
