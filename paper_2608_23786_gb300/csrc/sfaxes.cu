@@ -32,7 +32,7 @@ int sf_blocks(int N) { return 152 * (N < 64 ? 2 : 6); }
 __global__ void __launch_bounds__(kThreads) k_sf_axes(const double* __restrict__ u, int N, int logN, int pmax,
                                                       double* __restrict__ partial)
 {
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     const int halfN = N / 2;
     const int L = kThreads / halfN > 0 ? kThreads / halfN : 1;  // lines per batch
     double* line = sm;                                          // [L][N]
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kThreads) k_sf_axes(const double* __restrict__
 __global__ void __launch_bounds__(kThreads) k_sf_axes_f32(const double* __restrict__ u, int N, int logN,
                                                           double* __restrict__ partial)
 {
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     const int halfN = N / 2;
     const int L = kThreads / halfN > 0 ? kThreads / halfN : 1;
     float* line = reinterpret_cast<float*>(sm);  // [L][2 N]: each line twice, so that x + r needs no wrap

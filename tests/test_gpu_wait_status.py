@@ -78,3 +78,21 @@ def test_gradient_reports_it():
     ens.init()
     mclbm.mclbm_selftest_timeout(ens.ctx)
     assert _status(lambda: mclbm.mclbm_grad(ens.ctx, 0, 16, 8, ptr, need, 2)) == "TIMEOUT"
+
+
+@pytest.mark.parametrize("lattice,N,M,pattern", [(19, 32, 7, "pull"), (19, 64, 9, "aa"), (27, 64, 2, "pull")])
+def test_a_launch_that_finds_the_word_set_ends_and_is_reported(lattice, N, M, pattern):
+    """The multi-step kernel's ways out: with the error word set its warps leave at their first long
+    wait, in whatever part of the work; the call ends, the state is reported, and the next run is whole."""
+    mclbm.load(build_if_missing=True, lattice=lattice)
+    make = lambda: Ensemble(N, M, Re=12.5 * N, Ma=1.6 / 64, pattern=pattern, lattice=lattice).init()  # noqa: E731
+    ref, ens = make(), make()
+    mclbm.mclbm_set_step_limit(ref.ctx, 1)
+    ref.step(40)
+    mclbm.mclbm_selftest_timeout(ens.ctx)
+    ens.step(40)
+    assert _status(lambda: ens.energy()) == "TIMEOUT"
+    ens.init().step(40)
+    assert _status(lambda: ens.energy()) == "OK"
+    assert mclbm.mclbm_get_step_launches(ens.ctx) == (2, 80)
+    assert all(torch.equal(ens.populations(m), ref.populations(m)) for m in range(M))
