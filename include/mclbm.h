@@ -370,9 +370,9 @@ MCLBM_API int mclbm_autotune(mclbm_ctx* ctx, int32_t trial_steps, int32_t* kind,
  * Sub-step s of a macro step advances each level with s % (S / substeps[l]) == 0, all
  * in one persistent launch.  With graphs enabled (default when the stream is not the
  * legacy default stream) one period of the schedule is captured into a CUDA graph
- * on first use and replayed.  Where the multi-step kernel of mclbm_step serves the levels
- * that hold the work and no shape was set, each level instead takes its steps of a call in
- * one launch of it (the same results).  The batch borrows the contexts; destroy it first. */
+ * on first use and replayed.  Where no shape was set and the sizes of the levels say that it is faster,
+ * each level instead takes its steps of a call by itself, in the multi-step kernel of mclbm_step
+ * where that serves it (the same results).  The batch borrows the contexts; destroy it first. */
 typedef struct mclbm_batch mclbm_batch;
 MCLBM_API int mclbm_batch_create(mclbm_ctx* const* levels, int32_t nlev, const int32_t* substeps, mclbm_batch** out);
 MCLBM_API void mclbm_batch_destroy(mclbm_batch* b);

@@ -7,8 +7,9 @@ reduction, nothing else), so evaluating J costs one forward run whether or not a
 backward pass follows.  Backward re-runs the ensemble from the saved parameters
 through mclbm_grad (forward with checkpoints, segment recomputation, the hand-written
 adjoint kernels, parameter reduction) and multiplies the incoming gradient by dJ/dX.
-Both use the same stepper launches, so J of the two runs is the same to the bit.  The
-parameters live on the host (they enter the library as host arrays).
+The stepper gives the same bits whatever launches a run's steps take, so J of the two runs
+is the same to the bit.  The parameters live on the host (they enter the library as host
+arrays).
 """
 import torch
 from torch.autograd.function import once_differentiable

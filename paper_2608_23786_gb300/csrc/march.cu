@@ -91,7 +91,12 @@ bool march_order(MarchArgs<E>& a, const mclbm_ctx* c, int vec, int64_t steps)
 }
 
 // Whether `steps` steps of a context run faster in the multi-step kernel than with a launch per step.
-// The kernel's start (counters, cooperative launch, fill and drain) costs about 11 us a call.
+// The kernel's start (counters, cooperative launch, fill and drain) costs about 11 us a call.  It fills the
+// SMs it runs on, so contexts on several streams take turns: two FP32 contexts of 32^3 x 3 on two streams
+// take 1.5 ms per 200 steps against 1.6 with a launch per step, four 3.1 against 2.5 from one host
+// thread and 1.9 from four (one 0.78 against 1.24); from 64^3 on the kernel is faster at any number.  A
+// launch of half the blocks leaves room for a second context but costs one alone 22% at 32^3, so
+// this is left to mclbm_set_step_limit.
 //
 // FP32 storage, whose launch per step is at the HBM bound: per step the kernel saves 1 to 2 us below
 // 2^16 nodes (4.2 against 2.6 to 3.8 us at 8^3 to 32^3), 3 us at 32^3 x 7 (8.3 against 5.0), 4 us at 64^3

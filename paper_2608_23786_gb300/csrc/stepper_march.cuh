@@ -31,8 +31,9 @@
 // is then written, and the slots it overwrites are no longer read.  The tile with the lowest position
 // in the order among the unfinished ones never waits, and a group of warps waits only when it has
 // finished every tile of its own before, so the launch makes progress as long as its blocks are
-// resident together (a cooperative launch).  Every wait is bounded in time and records
-// MCLBM_ERR_TIMEOUT.
+// resident together (a cooperative launch, which starts when all of them fit: with 20 SMs held by another
+// stream for 2.5 s it started then, and ended as usual).  Every wait is bounded, in time and in looks, and
+// records MCLBM_ERR_TIMEOUT, which the calls that return results report.
 //
 // Roles.  Eight warps of a block collide, in two groups of four that each work on their own tiles.
 // Of the four warps of the third warp group, two look at the counters of a group's next tile and hand
