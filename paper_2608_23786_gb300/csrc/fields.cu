@@ -173,16 +173,23 @@ __global__ void k_reduce_rows(const double* __restrict__ partial, int rows, int 
 // FP16 348 -> 156, 64^3 x 8 FP64 415 -> 369.  D3Q27 FP16, whose run of four and the one in flight do not
 // fit the registers, takes two nodes: 16^3 x 200 192 us with element loads, 243 with four nodes, 136 with
 // two; 64^3 x 64 369 -> 242 (two).
-// Stores: 16 bytes where both fields are aligned, but FP32 element by element: with the second form of
-// store in its kernel the loop over the samples runs slower (energies wanted, with / without: 64^3 x 64 304 /
-// 274 us, 64^3 x 16 118 / 107, 32^3 x 200 381 / 329; without energies 64^3 x 4 35.0 / 33.2, 256^3 x 2 962 / 974).
+// Mean and variance alone of FP64 rows that span warps (N > 64) are read element by element too where the
+// loads are shifted: the end elements of the vector form spill (D3Q27 636 bytes a thread).  128^3 x 16, pull: D3Q27
+// 6250 us (elements) against 6511, D3Q19 4205 against 4258; with energies the vector form is the faster one
+// (D3Q19 4636 against 5621 us).
+// Stores: 16 bytes where both fields are aligned, but element by element after loads by element, node by
+// node: with the second form of store in its kernel the FP32 loop over the samples runs slower (energies
+// wanted, with / without: 64^3 x 64 304 / 274 us, 64^3 x 16 118 / 107, 32^3 x 200 381 / 329; without energies 64^3 x 4 35.0 /
+// 33.2, 256^3 x 2 962 / 974).
 template <class E>
 constexpr int kRunVec = sizeof(E) == 2 && Q == 19 ? 4 : 2;
 template <class E>
 constexpr bool kRunScalar = sizeof(E) == 4;
 constexpr int kSampleChunk = 8;
+// Samples whose |u|^2 trees run together (their shuffles overlap; a last batch that is not full still runs
+// whole: FP64 256^3 x 2 4962 us in batches of four, 4784 in twos, 32^3 x 60 397 and 402, AA 64^3 x 48 2061 and 1838).
 template <class E>
-constexpr int kEnergyBatch = kRunScalar<E> ? 1 : 4;  // samples whose |u|^2 trees run together (their shuffles overlap)
+constexpr int kEnergyBatch = kRunScalar<E> ? 1 : (sizeof(E) == 8 && Q == 19 ? 2 : 4);
 template <class E>
 constexpr int kStatsThreads = kRunScalar<E> ? 256 : 128;
 
@@ -208,6 +215,7 @@ __global__ void __launch_bounds__(kStatsThreads<E>) k_stats_pass(const E* __rest
 {
     using C = typename Storage<E>::compute;
     constexpr int VEC = kRunVec<E>;
+    constexpr bool SCALAR = kRunScalar<E> || (sizeof(E) == 8 && MODE != 1 && !WRAP && !WANT_E);
     extern __shared__ double ered[];  // WANT_E: [M][warps of the block]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if constexpr (WANT_E) {
@@ -234,11 +242,11 @@ __global__ void __launch_bounds__(kStatsThreads<E>) k_stats_pass(const E* __rest
                 s1[a][k] = s2[a][k] = 0.0;
                 p1[a][k] = p2[a][k] = C(0);
             }
-        RawRun<E, VEC> raw[kRunScalar<E> ? 1 : Q];  // the next sample's loads are in flight while one is summed
-        if constexpr (!kRunScalar<E>) issue_all<E, VEC, MODE, WRAP>(lat, g, p, lane, raw);
+        RawRun<E, VEC> raw[SCALAR ? 1 : Q];  // the next sample's loads are in flight while one is summed
+        if constexpr (!SCALAR) issue_all<E, VEC, MODE, WRAP>(lat, g, p, lane, raw);
         for (int m = 0; m < M; ++m) {
             C f[Q][VEC];
-            if constexpr (kRunScalar<E>) {
+            if constexpr (SCALAR) {
                 gather_run<E, MODE>(lat + (int64_t)m * Q * g.n, g, rows, x0, f);
             } else {
                 finish_all<E, VEC, MODE, WRAP>(g, p, lane, raw, f);
@@ -281,7 +289,7 @@ __global__ void __launch_bounds__(kStatsThreads<E>) k_stats_pass(const E* __rest
                 for (int a = 0; a < 3; ++a)
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) {
-                        if constexpr (kRunScalar<E>) {
+                        if constexpr (SCALAR) {
                             s1[a][k] += (double)p1[a][k];
                             s2[a][k] += (double)p2[a][k];
                         } else {
@@ -324,25 +332,32 @@ __global__ void __launch_bounds__(kStatsThreads<E>) k_stats_pass(const E* __rest
                 }
             }
         }
+        const auto mean_of = [&](int a, int k) { return fma(s1[a][k], invM, (double)u0[a][k]) * uscale; };
+        const auto var_of = [&](int a, int k) { return fma(-s1[a][k] * invM, s1[a][k], s2[a][k]) * vscale; };
+        if constexpr (SCALAR) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
+            for (int k = 0; k < VEC; ++k)
 #pragma unroll
-            for (int k = 0; k < VEC; k += 2) {
-                double mv[2], vv[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    mv[h] = fma(s1[a][k + h], invM, (double)u0[a][k + h]) * uscale;
-                    vv[h] = fma(-s1[a][k + h] * invM, s1[a][k + h], s2[a][k + h]) * vscale;
+                for (int a = 0; a < 3; ++a) {
+                    mean[a * g.n + node + k] = mean_of(a, k);
+                    var[a * g.n + node + k] = var_of(a, k);
                 }
-                double *mo = mean + a * g.n + node + k, *vo = var + a * g.n + node + k;
-                if (!kRunScalar<E> && pairs) {
-                    vstore<double, 2>(mo, mv);
-                    vstore<double, 2>(vo, vv);
-                } else {  // FP32, or the caller's fields are not 16-byte aligned
-                    mo[0] = mv[0], mo[1] = mv[1];
-                    vo[0] = vv[0], vo[1] = vv[1];
+        } else {
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int k = 0; k < VEC; k += 2) {
+                    const double mv[2] = {mean_of(a, k), mean_of(a, k + 1)}, vv[2] = {var_of(a, k), var_of(a, k + 1)};
+                    double *mo = mean + a * g.n + node + k, *vo = var + a * g.n + node + k;
+                    if (pairs) {
+                        vstore<double, 2>(mo, mv);
+                        vstore<double, 2>(vo, vv);
+                    } else {  // the caller's fields are not 16-byte aligned
+                        mo[0] = mv[0], mo[1] = mv[1];
+                        vo[0] = vv[0], vo[1] = vv[1];
+                    }
                 }
-            }
+        }
     }
     if constexpr (WANT_E) {
         __syncthreads();
